@@ -130,6 +130,7 @@ struct Job {
   long long* key_out;
   long long* q_out;
   int bin_mask;
+  float miss_lim;              // a straight line that meets the cylinder beyond this |z| misses for certain
 };
 
 // optional listmode records of a job (kept out of Job, which the kernel

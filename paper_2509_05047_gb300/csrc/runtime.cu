@@ -993,9 +993,11 @@ static int make_job(psc_ctx* ctx, const psc_sim_args* a, Job& jb, int& lut_dtype
     return fail(PSC_EINVAL, "block must be a multiple of 32 in [32, 512], grid >= 0");
   const psc_phantom_desc& pd = ph->desc;
   const double R2 = sc->desc.radius * sc->desc.radius;
+  double rho2 = 0.0;
   for (int i = 0; i < 4; ++i) {
     const double x = pd.ox + ((i & 1) ? pd.nx * pd.dx : 0.0), y = pd.oy + ((i & 2) ? pd.ny * pd.dy : 0.0);
     if (!(x * x + y * y < R2)) return fail(PSC_EINVAL, "phantom grid reaches outside the detector cylinder");
+    rho2 = std::max(rho2, x * x + y * y);
   }
   std::memset(&jb, 0, sizeof jb);
   jb.sc = sc->params;
@@ -1036,6 +1038,17 @@ static int make_job(psc_ctx* ctx, const psc_sim_args* a, Job& jb, int& lut_dtype
   jb.first = a->first_history;
   jb.n = a->n_histories;
   jb.bin_mask = a->bin_mask ? a->bin_mask : PSC_BIN_SCATTER;
+  // |z| beyond which a photon that has not interacted is certain to miss the
+  // detector.  The kernel's z of the hit is off the exact line's by at most
+  // about kMaxStraightSteps roundings of the position (2^-23 of the geometry's
+  // scale L each), times tan(incidence), 3 for a grid within 0.95 of the
+  // radius: below 64 * 2^-23 * 3 * 2 L = 5e-5 L.  The margin is L / 512; a grid
+  // nearer to the cylinder gets none (nothing is skipped).
+  {
+    const double half = 0.5 * sc->desc.n_rings * sc->desc.ring_pitch;
+    const double zmax = std::max(std::fabs(pd.oz), std::fabs(pd.oz + pd.nz * pd.dz));
+    jb.miss_lim = rho2 <= 0.95 * 0.95 * R2 ? (float)(half + (sc->desc.radius + half + zmax) / 512.0) : INFINITY;
+  }
   jb.acc = (unsigned long long*)acc->data.p;
   jb.cls_out = a->cls_out;
   jb.key_out = (long long*)a->key_out;

@@ -62,7 +62,8 @@ enum : int {
   C_VOX, C_AZ, C_BZ, C_ASC,                                  // listmode records only
   kColdFields
 };
-// F_META = state | photon << 3 | stream << 4;  F_CNT = steps | interactions << 16;
+// F_META = state | photon << 3 | stream << 4 | kMetaNeeds | kMetaNextMiss;
+// F_CNT = steps | interactions << 16;
 // C_ACRG = crystal | ring << 16 | scattered << 31;  C_BCRG = crystal | ring << 16;
 // C_APOS, C_BPOS = tpos | apos << 16;  C_ASC = photon A's F_CNT >> 15;
 // listmode runs flag a Rayleigh interaction in bit 15 of F_CNT (steps stay below 2^15)
@@ -70,6 +71,27 @@ enum : int {
 __host__ __device__ constexpr uint32_t meta(int state, int photon, int stream) {
   return (uint32_t)state | (uint32_t)photon << 3 | (uint32_t)stream << 4;
 }
+// Production launches (kDebug false) only add weights: a history that cannot
+// reach the accumulator may end as soon as that is certain, and its photons
+// may be followed in either order (their streams are independent and the
+// coincidence is symmetric in them).  EMIT therefore intersects the emission
+// line with the detector cylinder once for both photons:
+//   - a photon whose straight line leaves the cylinder axially, by more than
+//     a margin far above the FP32 error of the tracked position, is lost
+//     unless it interacts (kMetaNeeds).  Likewise the second photon when
+//     the first arrived unscattered and trues are not binned.  Such a photon
+//     ends its history where it leaves the grid, without a detection pass;
+//   - the photon that is less likely to be detected goes first: the one
+//     flying towards the nearer axial end when a line misses, else the one
+//     with the longer way through the phantom.  On the torso 0.16 instead of
+//     0.25 second photons per history, 2.6 instead of 3.1 step visits, 0.33
+//     instead of 0.85 detection visits (counted with the FP64 oracle).
+// Measured on the paper-scale torso, 1e9 histories: 101.7 -> 88.9 ms; the same
+// scanner with gaps and energy resolution, 1e8: 12.32 -> 9.76 ms.
+constexpr uint32_t kMetaNeeds = 1u << 6;     // the photon in flight is lost unless it interacts
+constexpr uint32_t kMetaNextMiss = 1u << 7;  // the second photon's straight line misses
+// the margin covers positions after this many steps (make_job)
+constexpr uint32_t kMaxStraightSteps = 64;
 
 
 // 1 << s, and 0 for s >= 32 (the PTX shift clamps its amount to the width)
@@ -401,7 +423,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
         if (sec == kEscape) need = S.escape_words;  // energy blur, edge-crystal draws
         if (sec == kCoinc && !blur) need = 0;
         if (k + need > 4 * nb) {
-          const uint32_t hlo = U(F_HLO, g), hhi = U(F_HHI, g), stream = U(F_META, g) >> 4;
+          const uint32_t hlo = U(F_HLO, g), hhi = U(F_HHI, g), stream = (U(F_META, g) >> 4) & 3u;
           do {
             const uint4 b = philox4x32_10(make_uint4(hlo, hhi, nb, stream), key);
             const uint32_t w0 = 4 * nb;
@@ -442,7 +464,23 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
           float sp, cp;
           sincospif(2.0f * uni(6), &sp, &cp);
           const float st = sqrtf(fmaxf(0.0f, 1.0f - ct * ct));
-          const float dx = st * cp, dy = st * sp, dz = ct;
+          float dx = st * cp, dy = st * sp, dz = ct;  // photon A's direction, then the first photon's
+          uint32_t flags = meta(kStep, 0, 1);
+          if (!kDebug) {
+            // axial coordinates of the two straight hits, times a
+            const float a = dx * dx + dy * dy, b = ex * dx + ey * dy, c = ex * ex + ey * ey - S.r2;
+            const float sq = sqrtf(fmaxf(b * b - a * c, 0.0f)), za = ez * a, lim = J.miss_lim * a;
+            const bool miss_a = fabsf(za + (sq - b) * dz) > lim, miss_b = fabsf(za - (sq + b) * dz) > lim;
+            const bool b_first = (miss_a || miss_b) ? ez * dz < 0.0f : b > 0.0f;
+            if (b_first) {
+              dx = -dx;
+              dy = -dy;
+              dz = -dz;
+              flags = meta(kStep, 0, 2);
+            }
+            if (b_first ? miss_b : miss_a) flags |= kMetaNeeds;
+            if (b_first ? miss_a : miss_b) flags |= kMetaNextMiss;
+          }
           setC(C_E0X, g, ex);
           setC(C_E0Y, g, ey);
           setC(C_E0Z, g, ez);
@@ -461,12 +499,12 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
           U(F_CNT, g) = 0;
           U(F_K, g) = 0;
           U(F_NB, g) = 0;
-          U(F_META, g) = meta(kStep, 0, 1);
+          U(F_META, g) = flags;
         }
 
         // ---- one Woodcock step ----
         if (sec == kStep) {
-          bool moved = false, ended = false;
+          bool moved = false, ended = false, lost = false;
           const uint32_t cnt = U(F_CNT, g);
           if ((int)(cnt & 0x7fffu) >= kMaxSteps) {
             finish(g, kStepLimit, -1, 0);
@@ -489,7 +527,10 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
               const float fz = (qz - ph.oz) * ph.inv_dz;
               if (!(fx >= 0.0f && fx < (float)ph.nx && fy >= 0.0f && fy < (float)ph.ny && fz >= 0.0f &&
                     fz < (float)ph.nz)) {
-                U(F_META, g) = (m & ~7u) | kEscape;  // outside the grid is vacuum: straight to the detector
+                // outside the grid is vacuum: straight to the detector, unless the photon
+                // is certain to miss it (cnt below 2^16: it did not interact)
+                if (!kDebug && (m & kMetaNeeds) && cnt <= kMaxStraightSteps) lost = true;
+                else U(F_META, g) = (m & ~7u) | kEscape;
               } else {
                 moved = true;
                 const int ix = min((int)fx, ph.nx - 1);
@@ -517,7 +558,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
                   ended = true;
                 }
               }
-              if (ended) finish(g, kAbsorbed, -1, 0);
+              if (ended || lost) finish(g, kAbsorbed, -1, 0);  // (lost: production only, no class is recorded)
               else U(F_K, g) = k;
             }
           }
@@ -648,7 +689,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
           const uint32_t m = U(F_META, g);
           if (cls != kDetected) {
             finish(g, cls, -1, 0);
-          } else if (((m >> 3) & 1u) == 0) {  // photon A: keep it, launch photon B back to back
+          } else if (((m >> 3) & 1u) == 0) {  // the first photon: keep it, launch the other one back to back
             const uint32_t nint = U(F_CNT, g) >> 16;
             CU(C_ACRG, g) = (uint32_t)cr | (uint32_t)rg << 16 | (nint > 0 ? 1u << 31 : 0u);
             if (S.gap_mode) CU(C_APOS, g) = pos;
@@ -674,7 +715,8 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
             U(F_CNT, g) = 0;
             U(F_K, g) = 0;
             U(F_NB, g) = 0;
-            U(F_META, g) = meta(kStep, 1, 2);
+            const bool needs = !kDebug && ((m & kMetaNextMiss) || (nint == 0 && !(J.bin_mask & PSC_BIN_TRUES)));
+            U(F_META, g) = meta(kStep, 1, 3 - (int)((m >> 4) & 3u)) | (needs ? kMetaNeeds : 0u);
           } else if (cr == (int)(CU(C_ACRG, g) & 0xffffu)) {
             finish(g, kSameCrystal, -1, 0);
           } else {
