@@ -58,8 +58,8 @@ __device__ __forceinline__ long long dbg_idx(DebugRecord* rec, unsigned site, lo
 
 constexpr int kMaxMaterials = 8;
 constexpr int kMaxSteps = 4096;     // Woodcock steps per photon (safety bound)
+constexpr unsigned long long kMaxChunk = 1ull << 16;  // histories of a work item (a slot holds 16 bits of the index)
 constexpr int kMaxTries = 64;       // rejection-sampling tries, last proposal kept
-constexpr int kRingWords = 8;       // per-lane window of the current Philox sub-stream
 constexpr float kPolarEps = 1e-6f;  // |d_z| > 1 - eps: rotate about the z axis
 constexpr float kRestKeV = 511.0f;
 constexpr float kEmitKeV = 511.0f;
@@ -151,7 +151,7 @@ struct BatchParams {
   int n_jobs;
   unsigned long long* next_chunk;  // work counter, zero at launch
   unsigned long long* stats;       // kStatCount counters or nullptr
-  uint32_t* cold;                  // per-CTA slot fields kept out of shared memory
+  uint4* cold;                     // per-CTA slot fields kept out of shared memory
   DebugRecord* dbg;                // bounds-check record of the debug build
   ListmodeOut lm[kMaxJobs];
 };
@@ -197,9 +197,15 @@ __device__ __forceinline__ void rotate(float3& d, float c, float u) {
     return;
   }
   const float rr = sqrtf(1.0f - d.z * d.z);
-  const float nx = c * d.x + sn * (cp * d.x * d.z - sp * d.y) / rr;
-  const float ny = c * d.y + sn * (cp * d.y * d.z + sp * d.x) / rr;
-  const float nz = c * d.z - sn * cp * rr;
+  // the fused operations are written out, so that a direction's last bit does
+  // not depend on which products the compiler chooses to contract
+  float rc;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(rr));
+  const float tx = __fmul_rn(sn, __fmaf_rn(__fmul_rn(cp, d.x), d.z, -__fmul_rn(sp, d.y)));
+  const float ty = __fmul_rn(sn, __fmaf_rn(__fmul_rn(cp, d.y), d.z, __fmul_rn(sp, d.x)));
+  const float nx = __fmaf_rn(c, d.x, __fmul_rn(tx, rc));
+  const float ny = __fmaf_rn(c, d.y, __fmul_rn(ty, rc));
+  const float nz = __fmaf_rn(c, d.z, -__fmul_rn(__fmul_rn(sn, cp), rr));
   d = make_float3(nx, ny, nz);
 }
 

@@ -1126,7 +1126,7 @@ static int batch_impl(psc_ctx* ctx, const psc_sim_args* args, int32_t n, psc_sta
       Job& jb = bp.jobs[j];
       const unsigned long long parts = (unsigned long long)sc_in.chunks_per_cta * (unsigned long long)grid;
       const unsigned long long per = (jb.n + parts - 1) / parts;
-      jb.chunk = std::min<unsigned long long>(std::max<unsigned long long>(1024, sc_in.max_chunk),
+      jb.chunk = std::min<unsigned long long>(std::min(kMaxChunk, std::max<unsigned long long>(1024, sc_in.max_chunk)),
                                               std::max<unsigned long long>(1024, per));
       total += (jb.n + jb.chunk - 1) / jb.chunk;
       bp.chunk_end[j] = total;
@@ -1156,7 +1156,7 @@ static int batch_impl(psc_ctx* ctx, const psc_sim_args* args, int32_t n, psc_sta
       }
       ctx->cold.bytes = cold_bytes;
     }
-    bp.cold = (uint32_t*)ctx->cold.p;
+    bp.cold = (uint4*)ctx->cold.p;
     if (!cap) CK(cudaStreamWaitEvent(s, ctx->cold_done, 0), "order slot buffer users");
     CK(launch_transport(bp, dt, grid, block, smem, s), "transport kernel launch");
     last_grid = grid;

@@ -8,26 +8,25 @@
 //        -> ESCAPE -> COINC -> next history
 //
 // Each warp owns a pool of kSlotsPerWarp photon slots whose state lives in
-// shared memory (structure of arrays; the fields only emission, detection
-// and coincidence touch live in an L2-resident global buffer instead, which
-// leaves room for 32 warps per SM).  Every loop iteration the warp picks the
-// section that the most slots wait for (weighting sections by their cost
-// was measured slower, since it runs sections on fewer lanes), packs up to
-// 32 slots in that state onto its 32 lanes, and runs the section once.  With
-// twice as many slots as lanes the chosen section usually fills the warp,
-// where one history per lane left most lanes idle (the states of 32
-// histories spread over six sections).  The code holds a single copy of each
-// section, and one rejection-sampling try runs per iteration.  Pools stay
-// per warp, so warps never wait on each other: pools shared by two warps
-// (barrier-coupled) and larger pools (fewer resident warps) both measured
-// slower on this issue-bound loop.
+// shared memory (the fields only emission, detection and coincidence touch
+// live in an L2-resident global buffer instead, which leaves room for 32
+// warps per SM).  Every loop iteration the warp picks the section that the
+// most slots wait for (weighting sections by their cost was measured slower,
+// since it runs sections on fewer lanes), packs up to 32 slots in that state
+// onto its 32 lanes, and runs the section once.  With three times as many
+// slots as lanes the chosen section nearly fills the warp, where one history
+// per lane left most lanes idle (the states of 32 histories spread over six
+// sections).  The code holds a single copy of each section, and one
+// rejection-sampling try runs per iteration.  Pools stay per warp, so warps
+// never wait on each other: pools shared by two warps (barrier-coupled)
+// measured slower on this issue-bound loop.
 //
 // Random numbers: a history's sub-streams (0: emission + TOF blur, 1: photon
-// A, 2: photon B) are read through an 8-word window per slot; the only
-// Philox4x32-10 evaluation sits before the sections and appends one block
-// when the slot's next section needs more words than the window holds.  The
-// words consumed, and their order, are those of the per-history definition,
-// so results do not depend on the schedule, the slot or the lane.
+// A, 2: photon B) are read through the slot's copy of the stream's last
+// Philox block; a section that reads more words than are left draws one more
+// block (emission draws its two blocks itself).  The words consumed, and
+// their order, are those of the per-history definition, so results do not
+// depend on the schedule, the slot or the lane.
 //
 // A history adds one fixed-point weight to the int64 accumulator or nothing
 // (Sec. 2.2.3: weighted or discarded, never duplicated); lanes of a warp
@@ -41,36 +40,49 @@ enum : int {
   kDone = 7
 };
 
-constexpr int kSlotsPerWarp = 64;
+// Slots per warp: the fuller the sections run, the fewer iterations a history
+// takes.  A model of the pool at the torso's section visits gives 0.204
+// iterations per history at 64 slots, 0.188 at 72 and 0.162 at 96 (0.155 at
+// 128, where every section fills 32 lanes).  96 is what 15 words a slot leave
+// room for beside the tables at 32 warps per SM.
+constexpr int kSlotsPerWarp = 96;
+constexpr int kSlotsPerLane = kSlotsPerWarp / 32;
 
-// fields of a photon slot kept in shared memory (used by every section):
-// field f of slot g at slots[f * n_slots + g]
-enum : int {
-  F_PX, F_PY, F_PZ, F_DX, F_DY, F_DZ, F_E, F_PATH,          // the photon in flight
-  F_K, F_NB, F_HLO, F_HHI, F_META, F_CNT, F_TRIES,          // stream position, history, state
-  F_RING,                                                    // kRingWords words of the sub-stream
-  kFields = F_RING + kRingWords
-};
-// fields read and written only at emission, detection and coincidence, kept
-// in an L2-resident global buffer: field f of slot g of CTA b at
-// cold[(b * kColdFields + f) * n_slots + g]
-enum : int {
-  C_E0X, C_E0Y, C_E0Z, C_D0X, C_D0Y, C_D0Z,                 // emission point, photon A direction
-  C_ACRG, C_AE, C_APATH, C_ANX, C_ANY, C_ADX, C_ADY, C_ADZ,  // photon A at the detector
-  C_BCRG, C_BNX, C_BNY,                                      // photon B at the detector
-  C_APOS, C_BPOS,                                            // LUT positions (scanners with gaps)
-  C_VOX, C_AZ, C_BZ, C_ASC,                                  // listmode records only
-  kColdFields
-};
-// F_META = state | photon << 3 | stream << 4 | kMetaNeeds | kMetaNextMiss;
-// F_CNT = steps | interactions << 16;
-// C_ACRG = crystal | ring << 16 | scattered << 31;  C_BCRG = crystal | ring << 16;
-// C_APOS, C_BPOS = tpos | apos << 16;  C_ASC = photon A's F_CNT >> 15;
-// listmode runs flag a Rayleigh interaction in bit 15 of F_CNT (steps stay below 2^15)
-// F_TRIES = tries (| material << 16 for a pending Rayleigh event)
+// A photon slot's state in shared memory, as arrays over the CTA's slots.
+// The loop is bound by issue slots, so a section moves its fields in 16-byte
+// accesses: 5 loads and 3 stores a Woodcock step.
+//   pos   {x, y, z, path}                        float4
+//   dir   {dx, dy, dz, energy}                   float4
+//   ring  the last Philox block of the stream    uint4
+//   kc    {stream position, counts}              uint2
+//   meta  section and flags (read by the vote)   uint32
+constexpr size_t kSlotBytes = 16 + 16 + 16 + 8 + 4;
+// kc.x = words left | blocks generated << 3 | rejection tries << 25: word i of
+// the section (i < words left) is ring[(i - left) & 3].  A section draws at
+// most one block, when fewer words are left than it reads, and then leaves at
+// most 4 of them unread.
+// kc.y = steps | interactions << 16; listmode runs flag a Rayleigh interaction
+// in bit 15 (steps stay below 2^15)
+constexpr uint32_t kKcBlock = 1u << 3, kKcTry = 1u << 25;
+__host__ __device__ constexpr uint32_t kc_left(uint32_t k) { return k & 7u; }
+// meta = section | photon << 3 | stream << 4 | kMetaNeeds | kMetaNextMiss |
+// material of a pending Rayleigh event << 8 | history of the work item << 16
 __host__ __device__ constexpr uint32_t meta(int state, int photon, int stream) {
   return (uint32_t)state | (uint32_t)photon << 3 | (uint32_t)stream << 4;
 }
+
+// fields written only at emission, detection and coincidence, in an
+// L2-resident global buffer: vector f of slot g of CTA b at
+// cold[(b * kColdVecs + f) * n_slots + g]
+enum : int {
+  C_E0,    // emission point, voxel (listmode)
+  C_D0,    // the first photon's emission direction, its path
+  C_A,     // first photon at the detector: crystal | ring << 16 | scattered << 31, energy, nx, ny
+  C_AD,    // its direction, its LUT position tpos | apos << 16 (scanners with gaps)
+  C_B,     // second photon: crystal | ring << 16, nx, ny, LUT position
+  C_LM,    // listmode: first photon's z, second photon's z, first photon's counts >> 15
+  kColdVecs
+};
 // Production launches (kDebug false) only add weights: a history that cannot
 // reach the accumulator may end as soon as that is certain, and its photons
 // may be followed in either order (their streams are independent and the
@@ -90,6 +102,7 @@ __host__ __device__ constexpr uint32_t meta(int state, int photon, int stream) {
 // scanner with gaps and energy resolution, 1e8: 12.32 -> 9.76 ms.
 constexpr uint32_t kMetaNeeds = 1u << 6;     // the photon in flight is lost unless it interacts
 constexpr uint32_t kMetaNextMiss = 1u << 7;  // the second photon's straight line misses
+constexpr int kMetaMaterial = 8, kMetaHistory = 16;
 // the margin covers positions after this many steps (make_job)
 constexpr uint32_t kMaxStraightSteps = 64;
 
@@ -259,27 +272,27 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
   extern __shared__ float4 smem[];
   const unsigned tid = threadIdx.x, bdim = blockDim.x;
   const int n_slots = kFixed ? 16 * kSlotsPerWarp : (int)(bdim >> 5) * kSlotsPerWarp;
-  uint32_t* slots = reinterpret_cast<uint32_t*>(smem);  // [kFields][n_slots]
-  float4* s_xs = reinterpret_cast<float4*>(slots + kFields * n_slots);
+  float4* s_pos = smem;
+  float4* s_dir = s_pos + n_slots;
+  uint4* s_ring = reinterpret_cast<uint4*>(s_dir + n_slots);
+  uint2* s_kc = reinterpret_cast<uint2*>(s_ring + n_slots);
+  uint32_t* s_meta = reinterpret_cast<uint32_t*>(s_kc + n_slots);
+  float4* s_xs = reinterpret_cast<float4*>(s_meta + n_slots);  // the job's tables (n_slots is a multiple of 96)
   __shared__ int s_j;
   __shared__ unsigned long long s_lo;         // first history of the chunk
   __shared__ unsigned s_len, s_next;          // chunk length, next offset to hand out
   __shared__ unsigned long long s_cnt[kStatCount];
-  __shared__ int s_sel[16][32];               // per warp: slot of each lane this iteration
+  __shared__ uint16_t s_sel[16][32];          // per warp: slot of each lane this iteration
   for (int i = tid; i < kStatCount; i += bdim) s_cnt[i] = 0;
   const unsigned lane_id = tid & 31u;
   const int warp = (int)(tid >> 5);
-  const int g0 = warp * kSlotsPerWarp + (int)lane_id, g1 = g0 + 32;  // the slots this lane refills
+  const int g0 = warp * kSlotsPerWarp + (int)lane_id;  // this lane refills slots g0, g0 + 32, g0 + 64
   const bool stats = kDebug && B.stats != nullptr;
   int cached = -1;
-
-  auto U = [&](int f, int g) -> uint32_t& { return slots[f * n_slots + g]; };
-  auto Fv = [&](int f, int g) -> float { return __uint_as_float(slots[f * n_slots + g]); };
-  auto setF = [&](int f, int g, float v) { slots[f * n_slots + g] = __float_as_uint(v); };
-  uint32_t* cold = B.cold + (size_t)blockIdx.x * kColdFields * n_slots;
-  auto CU = [&](int f, int g) -> uint32_t& { return cold[f * n_slots + g]; };
-  auto Cv = [&](int f, int g) -> float { return __uint_as_float(cold[f * n_slots + g]); };
-  auto setC = [&](int f, int g, float v) { cold[f * n_slots + g] = __float_as_uint(v); };
+  uint4* cold = B.cold + (size_t)blockIdx.x * kColdVecs * n_slots;
+  auto setC = [&](int f, int g, float x, float y, float z, uint32_t w) {
+    cold[f * n_slots + g] = make_uint4(__float_as_uint(x), __float_as_uint(y), __float_as_uint(z), w);
+  };
 
   for (;;) {
     // ---- fetch the next chunk of (job, history range) ----
@@ -342,23 +355,14 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
     // slot g takes the chunk's next history, or is done
     auto start = [&](int g) {
       const unsigned off = atomicAdd(&s_next, 1u);
-      if (off < s_len) {
-        const unsigned long long h = s_lo + off;
-        U(F_HLO, g) = (uint32_t)h;
-        U(F_HHI, g) = (uint32_t)(h >> 32);
-        U(F_META, g) = meta(kEmit, 0, 0);
-        U(F_K, g) = 0;
-        U(F_NB, g) = 0;
-      } else {
-        U(F_META, g) = kDone;
-      }
+      s_meta[g] = off < s_len ? meta(kEmit, 0, 0) | off << kMetaHistory : (uint32_t)kDone;
     };
     // a history ends in slot g: record its class (and bin, weight), start the next
-    auto finish = [&](int g, int cls, long long key_out, long long q_out) {
-      const unsigned long long h = (unsigned long long)U(F_HHI, g) << 32 | U(F_HLO, g);
-      const unsigned long long i = (unsigned long long)dbg_idx(B.dbg, kSiteHistOut, (long long)(h - J.first),
-                                                               (long long)J.n);
+    auto finish = [&](int g, uint32_t m, int cls, long long key_out, long long q_out) {
       if (kDebug) {
+        const unsigned long long h = s_lo + (m >> kMetaHistory);
+        const unsigned long long i = (unsigned long long)dbg_idx(B.dbg, kSiteHistOut, (long long)(h - J.first),
+                                                                 (long long)J.n);
         if (J.cls_out) J.cls_out[i] = (int8_t)cls;
         if (J.key_out) J.key_out[i] = key_out;
         if (J.q_out) J.q_out[i] = q_out;
@@ -367,30 +371,29 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
       start(g);
     };
 
-    start(g0);
-    start(g1);
+#pragma unroll
+    for (int i = 0; i < kSlotsPerLane; ++i) start(g0 + 32 * i);
     __syncwarp();
 
-    // words a section reads, one nibble per section: 7, 2, 4, 3, 0, 2.  After a refill
-    // the window holds words [4 nb - kRingWords, 4 nb) with 4 nb < k + need + 4, so it
-    // still holds word k only for need <= kRingWords - 3; EMIT (7) starts at k = 0.
-    // Detection reads at most 4 (energy blur 2, edge draws 2).
-    constexpr uint32_t kNeedNibbles = 0x203427u;
-    static_assert(((kNeedNibbles >> 4) & 15u) <= kRingWords - 3 && ((kNeedNibbles >> 8) & 15u) <= kRingWords - 3 &&
-                      ((kNeedNibbles >> 12) & 15u) <= kRingWords - 3 && ((kNeedNibbles >> 20) & 15u) <= kRingWords - 3 &&
-                      4 <= kRingWords - 3 && (kNeedNibbles & 15u) <= kRingWords,
-                  "a section's words must fit the Philox window");
+    // words a section reads of its stream, one nibble per section: (EMIT draws its own),
+    // 2, 4, 3, 0, 2.  Detection reads S.escape_words (energy blur 2, edge draws 2), at
+    // most 4: one block always covers what the ring lacks.
+    constexpr uint32_t kNeedNibbles = 0x203420u;
 
     for (;;) {
-      const int st0 = (int)(U(F_META, g0) & 7u), st1 = (int)(U(F_META, g1) & 7u);
-
       // ---- warp vote: the section that the most slots wait for ----
-      // slot counts per state, one byte each (at most 64 slots): states 0..3
+      // slot counts per state, one byte each (at most 96 slots): states 0..3
       // in lo, 4..7 in hi (sections 4, 5 in its bytes 0, 1), summed over the
       // warp by two reductions.  A state's bit is 1 << 8 st, or 1 << (8 st - 32)
       // in hi, where shift amounts of 32 and more (unsigned wrap included) give 0.
-      const unsigned lo = shl_or_zero(8u * st0) + shl_or_zero(8u * st1);
-      const unsigned hi = shl_or_zero(8u * st0 - 32u) + shl_or_zero(8u * st1 - 32u);
+      int st[kSlotsPerLane];
+      unsigned lo = 0, hi = 0;
+#pragma unroll
+      for (int i = 0; i < kSlotsPerLane; ++i) {
+        st[i] = (int)(s_meta[g0 + 32 * i] & 7u);
+        lo += shl_or_zero(8u * st[i]);
+        hi += shl_or_zero(8u * st[i] - 32u);
+      }
       const unsigned clo = __reduce_add_sync(0xffffffffu, lo), chi = __reduce_add_sync(0xffffffffu, hi);
       if ((clo | (chi & 0xffffu)) == 0u) break;  // every slot is done
       // the most-populated section, the lowest on a tie: keys count << 3 | (7 - q)
@@ -400,48 +403,64 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
       const unsigned k23 = __byte_perm(clo, 0u, 0x4342) * 8u + 0x00040005u;
       const unsigned k45 = __byte_perm(chi, 0u, 0x4140) * 8u + 0x00020003u;
       const unsigned km = umax16x2(umax16x2(k01, k23), k45);
-      const int sec = 7 - (int)(max(km & 0xffffu, km >> 16) & 7u);
-      const unsigned sm0 = __ballot_sync(0xffffffffu, st0 == sec);
-      const unsigned sm1 = __ballot_sync(0xffffffffu, st1 == sec);
+      const unsigned kmax = max(km & 0xffffu, km >> 16);
+      const int sec = 7 - (int)(kmax & 7u);
       // ---- pack up to 32 slots in that state onto the lanes ----
       const unsigned below = (1u << lane_id) - 1u;
-      const int n0 = __popc(sm0);
-      if (st0 == sec) s_sel[warp][__popc(sm0 & below)] = g0;
-      if (st1 == sec) {
-        const int r = n0 + __popc(sm1 & below);
-        if (r < 32) s_sel[warp][r] = g1;
+      int n = 0;
+#pragma unroll
+      for (int i = 0; i < kSlotsPerLane; ++i) {
+        const unsigned mask = __ballot_sync(0xffffffffu, st[i] == sec);
+        const int r = n + __popc(mask & below);
+        if (st[i] == sec && r < 32) s_sel[warp][r] = (uint16_t)(g0 + 32 * i);
+        n += __popc(mask);
       }
       __syncwarp();
-      const int g = (int)lane_id < min(32, n0 + __popc(sm1))
-                        ? (int)dbg_idx(B.dbg, kSiteSlot, s_sel[warp][lane_id], n_slots) : -1;
+      const int g = lane_id < (kmax >> 3) ? (int)dbg_idx(B.dbg, kSiteSlot, s_sel[warp][lane_id], n_slots) : -1;
       __syncwarp();
 
       if (g >= 0) {
-        // ---- refill the slot's window: the single Philox evaluation ----
-        uint32_t k = U(F_K, g), nb = U(F_NB, g);
-        int need = (int)((kNeedNibbles >> (4 * sec)) & 15u);
-        if (sec == kEscape) need = S.escape_words;  // energy blur, edge-crystal draws
-        if (sec == kCoinc && !blur) need = 0;
-        if (k + need > 4 * nb) {
-          const uint32_t hlo = U(F_HLO, g), hhi = U(F_HHI, g), stream = (U(F_META, g) >> 4) & 3u;
-          do {
-            const uint4 b = philox4x32_10(make_uint4(hlo, hhi, nb, stream), key);
-            const uint32_t w0 = 4 * nb;
-            U(F_RING + ((w0 + 0) & (kRingWords - 1)), g) = b.x;
-            U(F_RING + ((w0 + 1) & (kRingWords - 1)), g) = b.y;
-            U(F_RING + ((w0 + 2) & (kRingWords - 1)), g) = b.z;
-            U(F_RING + ((w0 + 3) & (kRingWords - 1)), g) = b.w;
-            ++nb;
-            count(true, kStatRng);
-          } while (k + need > 4 * nb);
-          U(F_NB, g) = nb;
+        const uint32_t m = s_meta[g];
+        auto history = [&]() -> unsigned long long { return s_lo + (m >> kMetaHistory); };
+        auto block = [&](uint32_t nb, uint32_t stream) -> uint4 {
+          const unsigned long long h = history();
+          count(true, kStatRng);
+          return philox4x32_10(make_uint4((uint32_t)h, (uint32_t)(h >> 32), nb, stream), key);
+        };
+        // ---- the section's random words r0 .. r3, from the ring and a new block ----
+        uint2 kc = make_uint2(0u, 0u);
+        uint32_t r0 = 0, r1 = 0, r2 = 0, r3 = 0;
+        if (sec != kEmit) {
+          kc = s_kc[g];
+          uint32_t need = (kNeedNibbles >> (4 * sec)) & 15u;
+          if (sec == kEscape) need = S.escape_words;  // energy blur, edge-crystal draws
+          if (sec == kCoinc && !blur) need = 0;
+          if (need) {
+            const uint32_t left = kc_left(kc.x);
+            const uint32_t* ring = reinterpret_cast<const uint32_t*>(s_ring + g);
+            r0 = ring[(0u - left) & 3u];
+            r1 = ring[(1u - left) & 3u];
+            if (need > 2) {
+              r2 = ring[(2u - left) & 3u];
+              r3 = ring[(3u - left) & 3u];
+            }
+            if (left < need) {  // word i >= left is word i - left of the new block
+              const uint4 b = block((kc.x >> 3) & 0x3fffffu, (m >> 4) & 3u);
+              s_ring[g] = b;
+              kc.x += kKcBlock + 4u;
+              r3 = left == 0 ? b.w : left == 1 ? b.z : left == 2 ? b.y : b.x;
+              r2 = left == 0 ? b.z : left == 1 ? b.y : left == 2 ? b.x : r2;
+              r1 = left == 0 ? b.y : left == 1 ? b.x : r1;
+              r0 = left == 0 ? b.x : r0;
+            }
+          }
         }
-        auto word = [&](uint32_t w) -> uint32_t { return U(F_RING + (w & (kRingWords - 1)), g); };
-        auto uni = [&](uint32_t w) -> float { return u01(word(w)); };
+        auto set_section = [&](int state) { s_meta[g] = (m & ~7u) | (uint32_t)state; };
 
         // ---- emission (stream 0, words 0..6) ----
         if (sec == kEmit) {
-          const uint32_t w0 = word(0), w1 = word(1);
+          const uint4 b0 = block(0, 0), b1 = block(1, 0);
+          const uint32_t w0 = b0.x, w1 = b0.y;
           const unsigned col = __umulhi(w0, (unsigned)ph.n_vox);  // n_vox < 2^31
           const uint2 at = __ldg(ph.alias + dbg_idx(B.dbg, kSiteAlias, col, ph.n_vox));
           const int v = ((w1 >> 9) < at.x) ? (int)col : (int)at.y;
@@ -458,11 +477,11 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
             ++iy;
             ix -= (unsigned)ph.nx;
           }
-          const float ex = ph.ox + ((float)ix + uni(2)) * ph.dx, ey = ph.oy + ((float)iy + uni(3)) * ph.dy,
-                      ez = ph.oz + ((float)iz + uni(4)) * ph.dz;
-          const float ct = 2.0f * uni(5) - 1.0f;
+          const float ex = ph.ox + ((float)ix + u01(b0.z)) * ph.dx, ey = ph.oy + ((float)iy + u01(b0.w)) * ph.dy,
+                      ez = ph.oz + ((float)iz + u01(b1.x)) * ph.dz;
+          const float ct = 2.0f * u01(b1.y) - 1.0f;
           float sp, cp;
-          sincospif(2.0f * uni(6), &sp, &cp);
+          sincospif(2.0f * u01(b1.z), &sp, &cp);
           const float st = sqrtf(fmaxf(0.0f, 1.0f - ct * ct));
           float dx = st * cp, dy = st * sp, dz = ct;  // photon A's direction, then the first photon's
           uint32_t flags = meta(kStep, 0, 1);
@@ -481,44 +500,37 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
             if (b_first ? miss_b : miss_a) flags |= kMetaNeeds;
             if (b_first ? miss_a : miss_b) flags |= kMetaNextMiss;
           }
-          setC(C_E0X, g, ex);
-          setC(C_E0Y, g, ey);
-          setC(C_E0Z, g, ez);
-          setC(C_D0X, g, dx);
-          setC(C_D0Y, g, dy);
-          setC(C_D0Z, g, dz);
-          if (kDebug && lm.out) CU(C_VOX, g) = (uint32_t)v;
-          setF(F_PX, g, ex);
-          setF(F_PY, g, ey);
-          setF(F_PZ, g, ez);
-          setF(F_DX, g, dx);
-          setF(F_DY, g, dy);
-          setF(F_DZ, g, dz);
-          setF(F_E, g, kEmitKeV);
-          setF(F_PATH, g, 0.0f);
-          U(F_CNT, g) = 0;
-          U(F_K, g) = 0;
-          U(F_NB, g) = 0;
-          U(F_META, g) = flags;
+          setC(C_E0, g, ex, ey, ez, (uint32_t)v);
+          setC(C_D0, g, dx, dy, dz, 0u);
+          s_pos[g] = make_float4(ex, ey, ez, 0.0f);
+          s_dir[g] = make_float4(dx, dy, dz, kEmitKeV);
+          s_kc[g] = make_uint2(0u, 0u);
+          s_meta[g] = flags | (m & 0xffff0000u);
         }
 
         // ---- one Woodcock step ----
         if (sec == kStep) {
           bool moved = false, ended = false, lost = false;
-          const uint32_t cnt = U(F_CNT, g);
+          const uint32_t cnt = kc.y;
           if ((int)(cnt & 0x7fffu) >= kMaxSteps) {
-            finish(g, kStepLimit, -1, 0);
+            finish(g, m, kStepLimit, -1, 0);
           } else {
-            const float e = Fv(F_E, g);
+            const float4 pos = s_pos[g], dir = s_dir[g];
+            const float e = dir.w;
             const float mu_max = interp_scalar(s_maj, ph.n_tab, ph.e0, e);
-            const uint32_t m = U(F_META, g);
             if (!(mu_max > 0.0f)) {
-              U(F_META, g) = (m & ~7u) | kEscape;
+              // no word was read: with 5 of them left, the ring lacks the oldest; drop the block again
+              if (kc_left(kc.x) > 4u) {
+                reinterpret_cast<uint32_t*>(s_ring + g)[3] = r0;
+                kc.x -= kKcBlock + 4u;
+              }
+              s_kc[g].x = kc.x;
+              set_section(kEscape);
             } else {
-              const float px = Fv(F_PX, g), py = Fv(F_PY, g), pz = Fv(F_PZ, g);
-              const float dx = Fv(F_DX, g), dy = Fv(F_DY, g), dz = Fv(F_DZ, g);
-              const float dist = -__logf(uni(k)) / mu_max;
-              ++k;
+              const float px = pos.x, py = pos.y, pz = pos.z;
+              const float dx = dir.x, dy = dir.y, dz = dir.z;
+              const float dist = -__logf(u01(r0)) / mu_max;
+              --kc.x;
               const float qx = px + dist * dx;
               const float qy = py + dist * dy;
               const float qz = pz + dist * dz;
@@ -530,36 +542,32 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
                 // outside the grid is vacuum: straight to the detector, unless the photon
                 // is certain to miss it (cnt below 2^16: it did not interact)
                 if (!kDebug && (m & kMetaNeeds) && cnt <= kMaxStraightSteps) lost = true;
-                else U(F_META, g) = (m & ~7u) | kEscape;
+                else set_section(kEscape);
               } else {
                 moved = true;
                 const int ix = min((int)fx, ph.nx - 1);
                 const int iy = min((int)fy, ph.ny - 1);
                 const int iz = min((int)fz, ph.nz - 1);
-                setF(F_PX, g, qx);
-                setF(F_PY, g, qy);
-                setF(F_PZ, g, qz);
-                setF(F_PATH, g, Fv(F_PATH, g) + dist);
-                U(F_CNT, g) = cnt + 1u;
+                s_pos[g] = make_float4(qx, qy, qz, pos.w + dist);
+                kc.y = cnt + 1u;
                 const float2 vx = __ldg(ph.vox + dbg_idx(B.dbg, kSiteVoxel, (unsigned)((iz * ph.ny + iy) * ph.nx + ix),
                                                          ph.n_vox));  // n_vox < 2^31
                 const int mat = (int)dbg_idx(B.dbg, kSiteMaterial, __float_as_int(vx.y), ph.n_mat);
                 const float4 cum = interp_xs(s_xs + mat * ph.n_tab, ph.n_tab, ph.e0, e);
-                const float t = uni(k) * mu_max;
-                ++k;
+                const float t = u01(r1) * mu_max;
+                --kc.x;
                 if (t < vx.x * cum.x) {
-                  U(F_META, g) = (m & ~7u) | kCompton;
-                  U(F_TRIES, g) = 0;
+                  set_section(kCompton);
                 } else if (t < vx.x * cum.y) {
-                  U(F_META, g) = (m & ~7u) | kRayleigh;
-                  U(F_TRIES, g) = (uint32_t)mat << 16;  // the material id travels with the pending event
+                  // the material id travels with the pending event
+                  s_meta[g] = (m & ~(7u | 7u << kMetaMaterial)) | kRayleigh | (uint32_t)mat << kMetaMaterial;
                 } else if (t < vx.x * cum.z) {
                   count(true, kStatPhoto);
                   ended = true;
                 }
               }
-              if (ended || lost) finish(g, kAbsorbed, -1, 0);  // (lost: production only, no class is recorded)
-              else U(F_K, g) = k;
+              if (ended || lost) finish(g, m, kAbsorbed, -1, 0);  // (lost: production only, no class is recorded)
+              else s_kc[g] = kc;
             }
           }
           count(moved, kStatSteps);
@@ -567,80 +575,73 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
 
         // ---- one Klein-Nishina try (Kahn's method on x = E/E') ----
         if (sec == kCompton) {
-          const float r1 = uni(k), r2 = uni(k + 1), r3 = uni(k + 2);
-          k += 3;
-          const uint32_t tries = U(F_TRIES, g) + 1u;
-          const float e = Fv(F_E, g);
+          const float u1 = u01(r0), u2 = u01(r1), u3 = u01(r2);
+          kc.x -= 3u;
+          const uint32_t tries = (kc.x >> 25) + 1u;
+          const float4 dir = s_dir[g];
+          const float e = dir.w;
           const float a = e / kRestKeV;
           const float two_a = 2.0f * a;
           float x, c;
           bool accept;
-          if (r1 < (1.0f + two_a) / (9.0f + two_a)) {
-            x = 1.0f + two_a * r2;
+          if (u1 < (1.0f + two_a) / (9.0f + two_a)) {
+            x = 1.0f + two_a * u2;
             c = 1.0f - (x - 1.0f) / a;
-            accept = r3 < 4.0f * (1.0f / x - 1.0f / (x * x));
+            accept = u3 < 4.0f * (1.0f / x - 1.0f / (x * x));
           } else {
-            x = (1.0f + two_a) / (1.0f + two_a * r2);
+            x = (1.0f + two_a) / (1.0f + two_a * u2);
             c = 1.0f - (x - 1.0f) / a;
-            accept = r3 < 0.5f * (c * c + 1.0f / x);
+            accept = u3 < 0.5f * (c * c + 1.0f / x);
           }
           count(true, kStatTries);
           if (accept || (int)tries >= kMaxTries) {
-            float3 d = make_float3(Fv(F_DX, g), Fv(F_DY, g), Fv(F_DZ, g));
-            rotate(d, c, uni(k));
-            ++k;
+            float3 d = make_float3(dir.x, dir.y, dir.z);
+            rotate(d, c, u01(r3));
             const float e1 = e / x;
             count(true, kStatCompton);
             if (e1 < S.e_kill) {
-              finish(g, kEnergyWindow, -1, 0);
+              finish(g, m, kEnergyWindow, -1, 0);
             } else {
-              setF(F_DX, g, d.x);
-              setF(F_DY, g, d.y);
-              setF(F_DZ, g, d.z);
-              setF(F_E, g, e1);
-              U(F_CNT, g) += 1u << 16;
-              U(F_K, g) = k;
-              U(F_META, g) = (U(F_META, g) & ~7u) | kStep;
+              s_dir[g] = make_float4(d.x, d.y, d.z, e1);
+              s_kc[g] = make_uint2((kc.x & (kKcTry - 1u)) - 1u, kc.y + (1u << 16));
+              set_section(kStep);
             }
           } else {
-            U(F_TRIES, g) = tries;
-            U(F_K, g) = k;
+            s_kc[g].x = kc.x + kKcTry;
           }
         }
 
         // ---- one Rayleigh try (material id in the upper half of tries) ----
         if (sec == kRayleigh) {
-          const float u1 = uni(k), u2 = uni(k + 1);
-          k += 2;
-          const uint32_t tries = U(F_TRIES, g) + 1u;
-          const float e = Fv(F_E, g);
+          const float u1 = u01(r0), u2 = u01(r1);
+          kc.x -= 2u;
+          const uint32_t tries = (kc.x >> 25) + 1u;
+          const float4 dir = s_dir[g];
+          const float e = dir.w;
           const float er = e / kRestKeV;
-          const float b = s_kappa[dbg_idx(B.dbg, kSiteKappa, tries >> 16, ph.n_mat)] * er * er;
+          const float b = s_kappa[dbg_idx(B.dbg, kSiteKappa, (m >> kMetaMaterial) & 7u, ph.n_mat)] * er * er;
           const float sv = u1 / (1.0f + b * (1.0f - u1));
           const float c = 1.0f - 2.0f * sv;
           count(true, kStatTries);
-          if (u2 < 0.5f * (1.0f + c * c) || (int)(tries & 0xffffu) >= kMaxTries) {
-            float3 d = make_float3(Fv(F_DX, g), Fv(F_DY, g), Fv(F_DZ, g));
-            rotate(d, c, uni(k));
-            ++k;
+          if (u2 < 0.5f * (1.0f + c * c) || (int)tries >= kMaxTries) {
+            float3 d = make_float3(dir.x, dir.y, dir.z);
+            rotate(d, c, u01(r2));
             count(true, kStatRayleigh);
-            setF(F_DX, g, d.x);
-            setF(F_DY, g, d.y);
-            setF(F_DZ, g, d.z);
-            U(F_CNT, g) = (U(F_CNT, g) + (1u << 16)) | (kDebug ? 0x8000u : 0u);
-            U(F_META, g) = (U(F_META, g) & ~7u) | kStep;
+            s_dir[g] = make_float4(d.x, d.y, d.z, e);
+            s_kc[g] = make_uint2((kc.x & (kKcTry - 1u)) - 1u, (kc.y + (1u << 16)) | (kDebug ? 0x8000u : 0u));
+            set_section(kStep);
           } else {
-            U(F_TRIES, g) = tries;
+            s_kc[g].x = kc.x + kKcTry;
           }
-          U(F_K, g) = k;
         }
 
         // ---- the photon reaches the detector cylinder ----
         if (sec == kEscape) {
-          const float px = Fv(F_PX, g), py = Fv(F_PY, g), pz = Fv(F_PZ, g);
-          const float dx = Fv(F_DX, g), dy = Fv(F_DY, g), dz = Fv(F_DZ, g);
-          const float e = Fv(F_E, g);
-          float path = Fv(F_PATH, g);
+          const float4 pos4 = s_pos[g], dir = s_dir[g];
+          const float px = pos4.x, py = pos4.y, pz = pos4.z;
+          const float dx = dir.x, dy = dir.y, dz = dir.z;
+          const float e = dir.w;
+          float path = pos4.w;
           const float a = dx * dx + dy * dy;
           int cls = kDetected, cr = 0, rg = 0;
           uint32_t pos = 0;  // LUT position tpos | apos << 16 (scanners with gaps)
@@ -666,14 +667,15 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
               ny = hy / S.radius;
               float ed = e;  // the energy the window tests: blurred by the resolution, if any
               if (S.e_res_k > 0.0f) {
-                ed = e + S.e_res_k * sqrtf(e) * (sqrtf(-2.0f * __logf(uni(k))) * cospif(2.0f * uni(k + 1)));
-                k += 2;
+                ed = e + S.e_res_k * sqrtf(e) * (sqrtf(-2.0f * __logf(u01(r0))) * cospif(2.0f * u01(r1)));
               }
               if (ed < S.e_lo || ed > S.e_hi) cls = kEnergyWindow;
               if (S.gap_mode && cls == kDetected) {
                 // two words cover both edge draws (the axial one is the second only after a
-                // transaxial one); the window holds them since escape_words counts them
-                const float u0 = S.gap_mode == 2 ? uni(k) : 0.0f, u1 = S.gap_mode == 2 ? uni(k + 1) : 0.0f;
+                // transaxial one); escape_words counts them
+                const bool blurred = S.e_res_k > 0.0f;
+                const float u0 = S.gap_mode == 2 ? u01(blurred ? r2 : r0) : 0.0f,
+                            u1 = S.gap_mode == 2 ? u01(blurred ? r3 : r1) : 0.0f;
                 const unsigned long long r = place(S, phi, hz, dx, dy, dz, nx, ny, u0, u1);
                 if ((uint32_t)r >> 31) {
                   cls = kLostAxial;  // lost in a gap
@@ -686,118 +688,102 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
             }
           }
           count(cls == kDetected, kStatDetected);
-          const uint32_t m = U(F_META, g);
+          const uint32_t crg = (uint32_t)cr | (uint32_t)rg << 16;
           if (cls != kDetected) {
-            finish(g, cls, -1, 0);
+            finish(g, m, cls, -1, 0);
           } else if (((m >> 3) & 1u) == 0) {  // the first photon: keep it, launch the other one back to back
-            const uint32_t nint = U(F_CNT, g) >> 16;
-            CU(C_ACRG, g) = (uint32_t)cr | (uint32_t)rg << 16 | (nint > 0 ? 1u << 31 : 0u);
-            if (S.gap_mode) CU(C_APOS, g) = pos;
-            if (kDebug && lm.out) {
-              setC(C_AZ, g, hz_det);
-              CU(C_ASC, g) = U(F_CNT, g) >> 15;
-            }
-            setC(C_AE, g, e);
-            setC(C_APATH, g, path);
-            setC(C_ANX, g, nx);
-            setC(C_ANY, g, ny);
-            setC(C_ADX, g, dx);
-            setC(C_ADY, g, dy);
-            setC(C_ADZ, g, dz);
-            setF(F_PX, g, Cv(C_E0X, g));
-            setF(F_PY, g, Cv(C_E0Y, g));
-            setF(F_PZ, g, Cv(C_E0Z, g));
-            setF(F_DX, g, -Cv(C_D0X, g));
-            setF(F_DY, g, -Cv(C_D0Y, g));
-            setF(F_DZ, g, -Cv(C_D0Z, g));
-            setF(F_E, g, kEmitKeV);
-            setF(F_PATH, g, 0.0f);
-            U(F_CNT, g) = 0;
-            U(F_K, g) = 0;
-            U(F_NB, g) = 0;
+            const uint32_t nint = kc.y >> 16;
+            cold[C_A * n_slots + g] = make_uint4(crg | (nint > 0 ? 1u << 31 : 0u), __float_as_uint(e),
+                                                 __float_as_uint(nx), __float_as_uint(ny));
+            setC(C_AD, g, dx, dy, dz, pos);
+            if (kDebug && lm.out) cold[C_LM * n_slots + g] = make_uint4(__float_as_uint(hz_det), 0u, kc.y >> 15, 0u);
+            const uint4 e0 = cold[C_E0 * n_slots + g], d0 = cold[C_D0 * n_slots + g];
+            cold[C_D0 * n_slots + g].w = __float_as_uint(path);
+            s_pos[g] = make_float4(__uint_as_float(e0.x), __uint_as_float(e0.y), __uint_as_float(e0.z), 0.0f);
+            s_dir[g] = make_float4(-__uint_as_float(d0.x), -__uint_as_float(d0.y), -__uint_as_float(d0.z), kEmitKeV);
+            s_kc[g] = make_uint2(0u, 0u);
             const bool needs = !kDebug && ((m & kMetaNextMiss) || (nint == 0 && !(J.bin_mask & PSC_BIN_TRUES)));
-            U(F_META, g) = meta(kStep, 1, 3 - (int)((m >> 4) & 3u)) | (needs ? kMetaNeeds : 0u);
-          } else if (cr == (int)(CU(C_ACRG, g) & 0xffffu)) {
-            finish(g, kSameCrystal, -1, 0);
+            s_meta[g] = meta(kStep, 1, 3 - (int)((m >> 4) & 3u)) | (needs ? kMetaNeeds : 0u) | (m & 0xffff0000u);
+          } else if (cr == (int)(cold[C_A * n_slots + g].x & 0xffffu)) {
+            finish(g, m, kSameCrystal, -1, 0);
           } else {
-            CU(C_BCRG, g) = (uint32_t)cr | (uint32_t)rg << 16;
-            if (S.gap_mode) CU(C_BPOS, g) = pos;
-            if (kDebug && lm.out) setC(C_BZ, g, hz_det);
-            setC(C_BNX, g, nx);
-            setC(C_BNY, g, ny);
-            setF(F_PATH, g, path);
-            if (blur) {  // the TOF blur reads stream 0, block 2
-              U(F_META, g) = meta(kCoinc, 1, 0);
-              U(F_K, g) = 8;
-              U(F_NB, g) = 2;
-            } else {
-              U(F_META, g) = meta(kCoinc, 1, 2);
-            }
+            setC(C_B, g, nx, ny, __uint_as_float(crg), pos);
+            if (kDebug && lm.out) cold[C_LM * n_slots + g].y = __float_as_uint(hz_det);
+            s_pos[g].w = path;
+            // the TOF blur reads stream 0, block 2
+            s_kc[g].x = 2u * kKcBlock;
+            s_meta[g] = meta(kCoinc, 1, 0) | (m & 0xffff0000u);
           }
         }
 
         // ---- coincidence: TOF, LOR bin, LUT weight, accumulate ----
         if (sec == kCoinc) {
-          const uint32_t acrg = CU(C_ACRG, g), bcrg = CU(C_BCRG, g);
+          const uint4 ca = cold[C_A * n_slots + g], cad = cold[C_AD * n_slots + g], cb = cold[C_B * n_slots + g];
+          const float4 dir = s_dir[g];
+          const uint32_t acrg = ca.x, bcrg = cb.z;
           const int a_cr = (int)(acrg & 0xffffu), a_rg = (int)((acrg >> 16) & 0x7fffu);
           const int b_cr = (int)(bcrg & 0xffffu), b_rg = (int)(bcrg >> 16);
-          const float a_path = Cv(C_APATH, g), path = Fv(F_PATH, g);
+          const float a_path = __uint_as_float(cold[C_D0 * n_slots + g].w), path = s_pos[g].w;
+          const float a_e = __uint_as_float(ca.y), a_nx = __uint_as_float(ca.z), a_ny = __uint_as_float(ca.w);
+          const float3 a_d = make_float3(__uint_as_float(cad.x), __uint_as_float(cad.y), __uint_as_float(cad.z));
+          const float b_nx = __uint_as_float(cb.x), b_ny = __uint_as_float(cb.y);
           const bool a_first = a_cr < b_cr;
           float delta = 0.5f * (a_first ? a_path - path : path - a_path);
           if (blur) {
-            const float gs = sqrtf(-2.0f * logf(uni(8))) * cospif(2.0f * uni(9));
+            const float gs = sqrtf(-2.0f * logf(u01(r0))) * cospif(2.0f * u01(r1));
             delta += S.tof_sigma * gs;
           }
           const long long key_ = a_first ? bin_key(S, a_cr, b_cr, a_rg, b_rg, delta)
                                          : bin_key(S, b_cr, a_cr, b_rg, a_rg, delta);
-          const bool scattered = (acrg >> 31) != 0u || (U(F_CNT, g) >> 16) > 0u;
+          const bool scattered = (acrg >> 31) != 0u || (kc.y >> 16) > 0u;
           const int cls = key_ < 0 ? kOutOfRange : scattered ? kScatter : kTrue;
           const bool take = cls == kScatter ? (J.bin_mask & 1) : cls == kTrue ? (J.bin_mask & 2) : false;
           long long q = 0;
           if (key_ >= 0 && (take || (kDebug && (J.q_out || lm.out)))) {
             float aa, ab, ba, bb;
-            angles(Cv(C_ANX, g), Cv(C_ANY, g), make_float3(Cv(C_ADX, g), Cv(C_ADY, g), Cv(C_ADZ, g)), aa, ab);
-            angles(Cv(C_BNX, g), Cv(C_BNY, g), make_float3(Fv(F_DX, g), Fv(F_DY, g), Fv(F_DZ, g)), ba, bb);
+            angles(a_nx, a_ny, a_d, aa, ab);
+            angles(b_nx, b_ny, make_float3(dir.x, dir.y, dir.z), ba, bb);
             int a_tp = a_cr % S.module_t, a_ap = a_rg % S.module_a, b_tp = b_cr % S.module_t,
                 b_ap = b_rg % S.module_a;
             if (S.gap_mode) {
-              const uint32_t pa = CU(C_APOS, g), pb = CU(C_BPOS, g);
+              const uint32_t pa = cad.w, pb = cb.w;
               a_tp = (int)(pa & 0xffffu);
               a_ap = (int)(pa >> 16);
               b_tp = (int)(pb & 0xffffu);
               b_ap = (int)(pb >> 16);
             }
-            const float w = lut_prob<DT>(J.lut, Cv(C_AE, g), aa, ab, a_tp, a_ap, B.dbg) *
-                            lut_prob<DT>(J.lut, Fv(F_E, g), ba, bb, b_tp, b_ap, B.dbg);
+            const float w = lut_prob<DT>(J.lut, a_e, aa, ab, a_tp, a_ap, B.dbg) *
+                            lut_prob<DT>(J.lut, dir.w, ba, bb, b_tp, b_ap, B.dbg);
             q = __float2ll_rn(w * 4294967296.0f);
           }
           if (kDebug && lm.out) {
             const unsigned long long slot = atomicAdd(lm.count, 1ull);
             if (slot < lm.cap) {
               psc_listmode_event* r = lm.out + slot;
-              r->history = (unsigned long long)U(F_HHI, g) << 32 | U(F_HLO, g);
+              const uint4 clm = cold[C_LM * n_slots + g];
+              r->history = history();
               r->q = key_ < 0 ? 0 : q;
-              r->voxel = (int)CU(C_VOX, g);
+              r->voxel = (int)cold[C_E0 * n_slots + g].w;
               r->cls = cls;
               r->delta_mm = 0.5f * (a_path - path);
-              r->energy_kev[0] = Cv(C_AE, g);
-              r->energy_kev[1] = Fv(F_E, g);
-              float pa = atan2f(Cv(C_ANY, g), Cv(C_ANX, g)), pb = atan2f(Cv(C_BNY, g), Cv(C_BNX, g));
+              r->energy_kev[0] = a_e;
+              r->energy_kev[1] = dir.w;
+              float pa = atan2f(a_ny, a_nx), pb = atan2f(b_ny, b_nx);
               r->phi[0] = pa < 0.0f ? pa + 6.283185307179586f : pa;
               r->phi[1] = pb < 0.0f ? pb + 6.283185307179586f : pb;
-              r->z_mm[0] = Cv(C_AZ, g);
-              r->z_mm[1] = Cv(C_BZ, g);
-              r->dir[0][0] = Cv(C_ADX, g);
-              r->dir[0][1] = Cv(C_ADY, g);
-              r->dir[0][2] = Cv(C_ADZ, g);
-              r->dir[1][0] = Fv(F_DX, g);
-              r->dir[1][1] = Fv(F_DY, g);
-              r->dir[1][2] = Fv(F_DZ, g);
+              r->z_mm[0] = __uint_as_float(clm.x);
+              r->z_mm[1] = __uint_as_float(clm.y);
+              r->dir[0][0] = a_d.x;
+              r->dir[0][1] = a_d.y;
+              r->dir[0][2] = a_d.z;
+              r->dir[1][0] = dir.x;
+              r->dir[1][1] = dir.y;
+              r->dir[1][2] = dir.z;
               r->crystal[0] = a_cr;
               r->crystal[1] = b_cr;
               r->ring[0] = a_rg;
               r->ring[1] = b_rg;
-              const uint32_t sa = CU(C_ASC, g), sb = U(F_CNT, g) >> 15;
+              const uint32_t sa = clm.z, sb = kc.y >> 15;
               r->n_scatter[0] = (uint16_t)min(sa >> 1, 65535u);
               r->n_scatter[1] = (uint16_t)min(sb >> 1, 65535u);
               r->rayleigh[0] = (uint8_t)(sa & 1u);
@@ -823,7 +809,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
               atomicAdd(&s_cnt[kStatWeight], (unsigned long long)q);
             }
           }
-          finish(g, cls, key_, cls == kOutOfRange ? 0 : q);
+          finish(g, m, cls, key_, cls == kOutOfRange ? 0 : q);
         }
       }
       __syncwarp();  // slot updates are visible to the lanes that vote on them next
@@ -839,11 +825,11 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
 }
 
 size_t transport_cold_words(int grid, int block) {
-  return (size_t)grid * kColdFields * (size_t)(block / 32) * kSlotsPerWarp;
+  return (size_t)grid * kColdVecs * 4 * (size_t)(block / 32) * kSlotsPerWarp;
 }
 
 size_t transport_smem_bytes(const PhantomParams& ph, int block) {
-  return sizeof(uint32_t) * kFields * (size_t)(block / 32) * kSlotsPerWarp +
+  return kSlotBytes * (size_t)(block / 32) * kSlotsPerWarp +
          sizeof(float4) * (size_t)ph.n_mat * ph.n_tab + sizeof(float) * (ph.n_tab + kMaxMaterials);
 }
 
