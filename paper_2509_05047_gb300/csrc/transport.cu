@@ -352,13 +352,8 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
       const unsigned b = __ballot_sync(act, pred);
       if (b && lane_id == (unsigned)(__ffs(act) - 1)) atomicAdd(&s_cnt[slot], (unsigned long long)__popc(b));
     };
-    // slot g takes the chunk's next history, or is done
-    auto start = [&](int g) {
-      const unsigned off = atomicAdd(&s_next, 1u);
-      s_meta[g] = off < s_len ? meta(kEmit, 0, 0) | off << kMetaHistory : (uint32_t)kDone;
-    };
-    // a history ends in slot g: record its class (and bin, weight), start the next
-    auto finish = [&](int g, uint32_t m, int cls, long long key_out, long long q_out) {
+    // a listmode launch records the history that ends in a slot: its class, bin and weight
+    auto record = [&](uint32_t m, int cls, long long key_out, long long q_out) {
       if (kDebug) {
         const unsigned long long h = s_lo + (m >> kMetaHistory);
         const unsigned long long i = (unsigned long long)dbg_idx(B.dbg, kSiteHistOut, (long long)(h - J.first),
@@ -368,11 +363,11 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
         if (J.q_out) J.q_out[i] = q_out;
         if (stats) atomicAdd(&s_cnt[kStatClass0 + cls], 1ull);
       }
-      start(g);
     };
 
 #pragma unroll
-    for (int i = 0; i < kSlotsPerLane; ++i) start(g0 + 32 * i);
+    for (int i = 0; i < kSlotsPerLane; ++i) s_meta[g0 + 32 * i] = kEmit;
+    unsigned waiting = ~0u;  // without the EMIT count once the work item has handed out its last history
     __syncwarp();
 
     // words a section reads of its stream, one nibble per section: (EMIT draws its own),
@@ -394,8 +389,8 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
         lo += shl_or_zero(8u * st[i]);
         hi += shl_or_zero(8u * st[i] - 32u);
       }
-      const unsigned clo = __reduce_add_sync(0xffffffffu, lo), chi = __reduce_add_sync(0xffffffffu, hi);
-      if ((clo | (chi & 0xffffu)) == 0u) break;  // every slot is done
+      const unsigned clo = __reduce_add_sync(0xffffffffu, lo) & waiting, chi = __reduce_add_sync(0xffffffffu, hi);
+      if ((clo | (chi & 0xffffu)) == 0u) break;  // no slot holds a history, none is left to start
       // the most-populated section, the lowest on a tie: keys count << 3 | (7 - q)
       // in 16-bit halves, two paired maxima, then the larger half.  A section
       // with slots outranks every empty one (key >= 8), so sec is never empty.
@@ -420,7 +415,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
       __syncwarp();
 
       if (g >= 0) {
-        const uint32_t m = s_meta[g];
+        uint32_t m = s_meta[g];
         auto history = [&]() -> unsigned long long { return s_lo + (m >> kMetaHistory); };
         auto block = [&](uint32_t nb, uint32_t stream) -> uint4 {
           const unsigned long long h = history();
@@ -456,9 +451,17 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
           }
         }
         auto set_section = [&](int state) { s_meta[g] = (m & ~7u) | (uint32_t)state; };
+        // the slot's history ends: it waits in EMIT for the work item's next one
+        auto finish = [&](int cls, long long key_out, long long q_out) {
+          record(m, cls, key_out, q_out);
+          s_meta[g] = kEmit;
+        };
 
         // ---- emission (stream 0, words 0..6) ----
-        if (sec == kEmit) {
+        // (the slot takes the work item's next history, if there is one)
+        const unsigned off = sec == kEmit ? atomicAdd(&s_next, 1u) : ~0u;
+        if (off < s_len) {
+          m = off << kMetaHistory;
           const uint4 b0 = block(0, 0), b1 = block(1, 0);
           const uint32_t w0 = b0.x, w1 = b0.y;
           const unsigned col = __umulhi(w0, (unsigned)ph.n_vox);  // n_vox < 2^31
@@ -505,70 +508,63 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
           s_pos[g] = make_float4(ex, ey, ez, 0.0f);
           s_dir[g] = make_float4(dx, dy, dz, kEmitKeV);
           s_kc[g] = make_uint2(0u, 0u);
-          s_meta[g] = flags | (m & 0xffff0000u);
+          s_meta[g] = flags | m;
         }
 
         // ---- one Woodcock step ----
         if (sec == kStep) {
-          bool moved = false, ended = false, lost = false;
           const uint32_t cnt = kc.y;
+          const float4 pos = s_pos[g], dir = s_dir[g];
+          const float e = dir.w;
+          const float mu_max = interp_scalar(s_maj, ph.n_tab, ph.e0, e);
+          bool moved = false;
           if ((int)(cnt & 0x7fffu) >= kMaxSteps) {
-            finish(g, m, kStepLimit, -1, 0);
-          } else {
-            const float4 pos = s_pos[g], dir = s_dir[g];
-            const float e = dir.w;
-            const float mu_max = interp_scalar(s_maj, ph.n_tab, ph.e0, e);
-            if (!(mu_max > 0.0f)) {
-              // no word was read: with 5 of them left, the ring lacks the oldest; drop the block again
-              if (kc_left(kc.x) > 4u) {
-                reinterpret_cast<uint32_t*>(s_ring + g)[3] = r0;
-                kc.x -= kKcBlock + 4u;
-              }
-              s_kc[g].x = kc.x;
-              set_section(kEscape);
-            } else {
-              const float px = pos.x, py = pos.y, pz = pos.z;
-              const float dx = dir.x, dy = dir.y, dz = dir.z;
-              const float dist = -__logf(u01(r0)) / mu_max;
-              --kc.x;
-              const float qx = px + dist * dx;
-              const float qy = py + dist * dy;
-              const float qz = pz + dist * dz;
-              const float fx = (qx - ph.ox) * ph.inv_dx;
-              const float fy = (qy - ph.oy) * ph.inv_dy;
-              const float fz = (qz - ph.oz) * ph.inv_dz;
-              if (!(fx >= 0.0f && fx < (float)ph.nx && fy >= 0.0f && fy < (float)ph.ny && fz >= 0.0f &&
-                    fz < (float)ph.nz)) {
-                // outside the grid is vacuum: straight to the detector, unless the photon
-                // is certain to miss it (cnt below 2^16: it did not interact)
-                if (!kDebug && (m & kMetaNeeds) && cnt <= kMaxStraightSteps) lost = true;
-                else set_section(kEscape);
-              } else {
-                moved = true;
-                const int ix = min((int)fx, ph.nx - 1);
-                const int iy = min((int)fy, ph.ny - 1);
-                const int iz = min((int)fz, ph.nz - 1);
-                s_pos[g] = make_float4(qx, qy, qz, pos.w + dist);
-                kc.y = cnt + 1u;
-                const float2 vx = __ldg(ph.vox + dbg_idx(B.dbg, kSiteVoxel, (unsigned)((iz * ph.ny + iy) * ph.nx + ix),
-                                                         ph.n_vox));  // n_vox < 2^31
-                const int mat = (int)dbg_idx(B.dbg, kSiteMaterial, __float_as_int(vx.y), ph.n_mat);
-                const float4 cum = interp_xs(s_xs + mat * ph.n_tab, ph.n_tab, ph.e0, e);
-                const float t = u01(r1) * mu_max;
-                --kc.x;
-                if (t < vx.x * cum.x) {
-                  set_section(kCompton);
-                } else if (t < vx.x * cum.y) {
-                  // the material id travels with the pending event
-                  s_meta[g] = (m & ~(7u | 7u << kMetaMaterial)) | kRayleigh | (uint32_t)mat << kMetaMaterial;
-                } else if (t < vx.x * cum.z) {
-                  count(true, kStatPhoto);
-                  ended = true;
-                }
-              }
-              if (ended || lost) finish(g, m, kAbsorbed, -1, 0);  // (lost: production only, no class is recorded)
-              else s_kc[g] = kc;
+            finish(kStepLimit, -1, 0);
+          } else if (!(mu_max > 0.0f)) {
+            // no word was read: with 5 of them left, the ring lacks the oldest; drop the block again
+            if (kc_left(kc.x) > 4u) {
+              reinterpret_cast<uint32_t*>(s_ring + g)[3] = r0;
+              kc.x -= kKcBlock + 4u;
             }
+            s_kc[g].x = kc.x;
+            set_section(kEscape);
+          } else {
+            const float px = pos.x, py = pos.y, pz = pos.z;
+            const float dx = dir.x, dy = dir.y, dz = dir.z;
+            const float dist = -__logf(u01(r0)) / mu_max;
+            const float qx = px + dist * dx;
+            const float qy = py + dist * dy;
+            const float qz = pz + dist * dz;
+            const float fx = (qx - ph.ox) * ph.inv_dx;
+            const float fy = (qy - ph.oy) * ph.inv_dy;
+            const float fz = (qz - ph.oz) * ph.inv_dz;
+            // outside the grid is vacuum: straight to the detector, unless the photon
+            // is certain to miss it (cnt below 2^16: it did not interact)
+            int next = !kDebug && (m & kMetaNeeds) && cnt <= kMaxStraightSteps ? kEmit : kEscape;
+            --kc.x;
+            moved = fx >= 0.0f && fx < (float)ph.nx && fy >= 0.0f && fy < (float)ph.ny && fz >= 0.0f &&
+                    fz < (float)ph.nz;
+            if (moved) {
+              const int ix = min((int)fx, ph.nx - 1);
+              const int iy = min((int)fy, ph.ny - 1);
+              const int iz = min((int)fz, ph.nz - 1);
+              s_pos[g] = make_float4(qx, qy, qz, pos.w + dist);
+              const float2 vx = __ldg(ph.vox + dbg_idx(B.dbg, kSiteVoxel, (unsigned)((iz * ph.ny + iy) * ph.nx + ix),
+                                                       ph.n_vox));  // n_vox < 2^31
+              const int mat = (int)dbg_idx(B.dbg, kSiteMaterial, __float_as_int(vx.y), ph.n_mat);
+              const float4 cum = interp_xs(s_xs + mat * ph.n_tab, ph.n_tab, ph.e0, e);
+              const float t = u01(r1) * mu_max;
+              --kc.x;
+              kc.y = cnt + 1u;
+              next = t < vx.x * cum.x ? kCompton : t < vx.x * cum.y ? kRayleigh : t < vx.x * cum.z ? kEmit : kStep;
+              if (next == kEmit) {
+                count(true, kStatPhoto);
+                record(m, kAbsorbed, -1, 0);
+              }
+              m = (m & ~(7u << kMetaMaterial)) | (uint32_t)mat << kMetaMaterial;  // travels with a Rayleigh event
+            }
+            s_kc[g] = kc;
+            set_section(next);
           }
           count(moved, kStatSteps);
         }
@@ -594,21 +590,22 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
             accept = u3 < 0.5f * (c * c + 1.0f / x);
           }
           count(true, kStatTries);
+          kc.x += kKcTry;
           if (accept || (int)tries >= kMaxTries) {
-            float3 d = make_float3(dir.x, dir.y, dir.z);
-            rotate(d, c, u01(r3));
             const float e1 = e / x;
             count(true, kStatCompton);
+            kc.x = (kc.x & (kKcTry - 1u)) - 1u;
+            kc.y += 1u << 16;
             if (e1 < S.e_kill) {
-              finish(g, m, kEnergyWindow, -1, 0);
+              finish(kEnergyWindow, -1, 0);
             } else {
+              float3 d = make_float3(dir.x, dir.y, dir.z);
+              rotate(d, c, u01(r3));
               s_dir[g] = make_float4(d.x, d.y, d.z, e1);
-              s_kc[g] = make_uint2((kc.x & (kKcTry - 1u)) - 1u, kc.y + (1u << 16));
               set_section(kStep);
             }
-          } else {
-            s_kc[g].x = kc.x + kKcTry;
           }
+          s_kc[g] = kc;
         }
 
         // ---- one Rayleigh try (material id in the upper half of tries) ----
@@ -690,7 +687,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
           count(cls == kDetected, kStatDetected);
           const uint32_t crg = (uint32_t)cr | (uint32_t)rg << 16;
           if (cls != kDetected) {
-            finish(g, m, cls, -1, 0);
+            finish(cls, -1, 0);
           } else if (((m >> 3) & 1u) == 0) {  // the first photon: keep it, launch the other one back to back
             const uint32_t nint = kc.y >> 16;
             cold[C_A * n_slots + g] = make_uint4(crg | (nint > 0 ? 1u << 31 : 0u), __float_as_uint(e),
@@ -705,7 +702,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
             const bool needs = !kDebug && ((m & kMetaNextMiss) || (nint == 0 && !(J.bin_mask & PSC_BIN_TRUES)));
             s_meta[g] = meta(kStep, 1, 3 - (int)((m >> 4) & 3u)) | (needs ? kMetaNeeds : 0u) | (m & 0xffff0000u);
           } else if (cr == (int)(cold[C_A * n_slots + g].x & 0xffffu)) {
-            finish(g, m, kSameCrystal, -1, 0);
+            finish(kSameCrystal, -1, 0);
           } else {
             setC(C_B, g, nx, ny, __uint_as_float(crg), pos);
             if (kDebug && lm.out) cold[C_LM * n_slots + g].y = __float_as_uint(hz_det);
@@ -809,10 +806,11 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
               atomicAdd(&s_cnt[kStatWeight], (unsigned long long)q);
             }
           }
-          finish(g, m, cls, key_, cls == kOutOfRange ? 0 : q);
+          finish(cls, key_, cls == kOutOfRange ? 0 : q);
         }
       }
       __syncwarp();  // slot updates are visible to the lanes that vote on them next
+      if (sec == kEmit && s_next >= s_len) waiting = ~0xffu;
     }
 
     __syncthreads();  // every slot is done with the chunk before the next fetch
