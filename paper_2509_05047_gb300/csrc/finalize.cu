@@ -253,27 +253,124 @@ __device__ __forceinline__ long long plane_at(const FinParams& P, long long j) {
   }
 }
 
+// A normal double's significand (53 bits, hidden bit set) in two words, and
+// its unbiased exponent: value = hi:lo 2^(e - 52).
+struct Sig {
+  unsigned hi, lo;
+  int e;
+};
+
+__device__ __forceinline__ Sig sig_of(double d) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+  const unsigned hi = (unsigned)(u >> 32);
+  return Sig{(hi & 0xfffffu) | 0x100000u, (unsigned)u, (int)((hi >> 20) & 0x7ffu) - 1023};
+}
+
+// the product of two significands rounded to nearest even, from four 32 x 32-bit
+// products: the 106-bit product in words w3:w2:w1:w0, shifted up by one where it
+// lies below 2^105, its top 53 bits kept, the rest decides the rounding
+__device__ __forceinline__ Sig sig_mul(Sig a, Sig b) {
+  const unsigned long long t0 = (unsigned long long)a.lo * b.lo;
+  const unsigned long long t1 = (unsigned long long)a.hi * b.lo + (t0 >> 32);
+  const unsigned long long t2 = (unsigned long long)a.lo * b.hi + (unsigned)t1;
+  const unsigned long long t3 = (unsigned long long)a.hi * b.hi + (t1 >> 32) + (t2 >> 32);
+  unsigned w3 = (unsigned)(t3 >> 32), w2 = (unsigned)t3, w1 = (unsigned)t2, w0 = (unsigned)t0;
+  const unsigned top = w3 >> 9;  // 1: the product is at least 2^105
+  if (!top) {
+    w3 = __funnelshift_l(w2, w3, 1);
+    w2 = __funnelshift_l(w1, w2, 1);
+    w1 = __funnelshift_l(w0, w1, 1);
+    w0 <<= 1;
+  }
+  Sig r;
+  r.hi = __funnelshift_l(w2, w3, 11);
+  r.lo = __funnelshift_l(w1, w2, 11);
+  r.e = a.e + b.e + (int)top;
+  const unsigned rem = (w1 << 11) | (w0 != 0u ? 1u : 0u);
+  const unsigned up = (rem > 0x80000000u || (rem == 0x80000000u && (r.lo & 1u))) ? 1u : 0u;
+  r.lo += up;
+  r.hi += r.lo < up ? 1u : 0u;
+  if (r.hi >> 21) {  // rounded up to 2^53 (the low word is then 0)
+    r.hi = 0x100000u;
+    ++r.e;
+  }
+  return r;
+}
+
+__device__ __noinline__ double plain_bin_general(unsigned long long u, double c, double s, bool has_s) {
+  const double x = dmul(i64_to_f64((long long)u), c);
+  return has_s ? dmul(x, s) : x;
+}
+
 // ---------------------------------------------------------------------------
 // no smoothing: out = (acc * c) * sens (FP64)
+//
+// Two correctly rounded FP64 products a bin.  The FP64 pipe would take two to
+// three times as long as the memory, so the significands are multiplied on the
+// integer pipes without leaving their unpacked form (about 65 instructions a
+// bin; bins without an event, most of them, skip the products).  A thread has
+// four bins in flight, 256 apart: with one at a time and packed intermediates
+// (integer products of 64-bit halves, rounding by variable shifts) the kernel
+// waited on memory and on itself.  288 x 16 scanner, 13 TOF bins, per-LOR
+// sensitivity (137.5 M bins, 2.29 GB): 1330 -> 490 us with 2 % of the bins
+// filled, 1506 -> 756 us with all of them.
 // ---------------------------------------------------------------------------
+constexpr int kPlainBins = 4;
+
 __global__ void __launch_bounds__(256) finalize_plain_kernel(const __grid_constant__ FinParams P) {
   // grid.y = plane, grid.x strides over the plane's J = V * R * T bins
   const long long plane = plane_at(P, P.plane0 + (long long)blockIdx.y);
   const int J = P.V * P.R * P.T;
   const long long base = plane * J;
   const long long lor0 = plane * (long long)P.V * P.R;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < J; j += gridDim.x * blockDim.x) {
-    const long long i = dbg_idx(P.dbg, kSiteFinBin, base + j, P.n_bins);
-    double x = dmul(i64_to_f64(__ldg(P.acc + i)), P.c);
-    if (P.sens)
-      x = dmul(x, at(P.sens, P.sens_per_lor ? dbg_idx(P.dbg, kSiteFinLor, lor0 + fdiv((unsigned)j, P.magic_T),
-                                                      P.n_bins / P.T)
-                                            : i));
-    P.out[i] = x;
+  const long long* __restrict__ acc = P.acc + base;
+  double* __restrict__ out = P.out + base;
+  const double* __restrict__ sens = P.sens ? P.sens + (P.sens_per_lor ? lor0 : base) : nullptr;
+  const Sig c = sig_of(P.c);
+  const unsigned c_sign = (unsigned)((unsigned long long)__double_as_longlong(P.c) >> 32) & 0x80000000u;
+  const bool c_normal = c.e > -1023 && c.e < 1024;
+  for (int j0 = blockIdx.x * (256 * kPlainBins) + threadIdx.x; j0 < J; j0 += gridDim.x * (256 * kPlainBins)) {
+    unsigned long long u[kPlainBins];
+    double s[kPlainBins];
+#pragma unroll
+    for (int q = 0; q < kPlainBins; ++q) {
+      const int j = j0 + 256 * q;
+      u[q] = 0;
+      s[q] = 1.0;
+      if (j < J) {
+        u[q] = (unsigned long long)__ldg(acc + (dbg_idx(P.dbg, kSiteFinBin, base + j, P.n_bins) - base));
+        if (sens)
+          s[q] = __ldg(sens + (P.sens_per_lor ? dbg_idx(P.dbg, kSiteFinLor, lor0 + fdiv((unsigned)j, P.magic_T),
+                                                        P.n_bins / P.T) - lor0
+                                              : (long long)j));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kPlainBins; ++q) {
+      const int j = j0 + 256 * q;
+      if (j >= J) break;
+      const unsigned s_hi = (unsigned)((unsigned long long)__double_as_longlong(s[q]) >> 32);
+      const unsigned sign = c_sign ^ (s_hi & 0x80000000u);
+      const unsigned s_exp = (s_hi >> 20) & 0x7ffu;
+      double x;
+      if (u[q] == 0 && s_exp != 0x7ffu) {
+        x = __hiloint2double((int)sign, 0);
+      } else if ((u[q] >> 53) != 0 || u[q] == 0 || !c_normal || s_exp - 1u >= 0x7feu) {
+        x = plain_bin_general(u[q], P.c, s[q], sens != nullptr);
+      } else {
+        const int lz = __clzll((long long)u[q]);
+        const unsigned long long m = u[q] << (lz - 11);
+        Sig r = sig_mul(Sig{(unsigned)(m >> 32), (unsigned)m, 63 - lz}, c);
+        bool normal = r.e > -1023 && r.e < 1024;
+        if (sens) r = sig_mul(r, sig_of(s[q]));
+        normal = normal && r.e > -1023 && r.e < 1024;
+        x = __hiloint2double((int)(sign | (((unsigned)(r.e + 1022) << 20) + r.hi)), (int)r.lo);
+        if (!normal) x = plain_bin_general(u[q], P.c, s[q], sens != nullptr);
+      }
+      out[j] = x;
+    }
   }
 }
-
-
 
 // ---------------------------------------------------------------------------
 // the sliding window down one column of n rows; row r of the source is
@@ -890,7 +987,8 @@ cudaError_t launch_finalize_planes(const FinParams& p, int lo, int hi, int sms, 
   if (hi <= lo) return cudaSuccess;
   const long long J = (long long)p.V * p.R * p.T;
   const long long n = hi - lo;
-  const long long per_plane = std::max(1LL, std::min((J + 255) / 256, 8LL * sms / n + 1));
+  // a few thousand bins a CTA, or all of a plane's strides when the planes alone fill the chip
+  const long long per_plane = std::max(1LL, std::min((J + 256 * kPlainBins - 1) / (256 * kPlainBins), 64LL * sms / n + 1));
   FinParams q = p;
   q.plane0 = lo;
   finalize_plain_kernel<<<dim3((unsigned)per_plane, (unsigned)n), 256, 0, s>>>(q);
