@@ -121,60 +121,76 @@ __global__ void rotate_sum_kernel(const long long* __restrict__ in, long long* _
   out[(((long long)p * V + v) * R + r) * T + t] = sum;
 }
 
-// bin index of the LOR (a + c, b + c) mod n of plane (ra, rb) and TOF bin t:
-// when the order reverses, the rings swap and the TOF bin mirrors
-__device__ __forceinline__ long long rotated_bin(int n, int n_rings, int R, int T, int rad_off, int a2, int b2,
-                                                 int ra, int rb, int t) {
-  const bool flip = a2 > b2;
-  const int lo = flip ? b2 : a2, hi = flip ? a2 : b2;
-  int f = lo + hi, s = 1;
-  if (f >= n) {
-    f -= n;
-    s = -1;
-  }
-  const int v2 = f >> 1;
-  const int r2 = s * (n / 2 - (hi - lo)) + n / 2 - 1 - rad_off;
-  const long long p2 = flip ? (long long)rb * n_rings + ra : (long long)ra * n_rings + rb;
-  const int t2 = flip ? T - 1 - t : t;
-  return ((p2 * (n / 2) + v2) * R + r2) * T + t2;
-}
-
 // The same sum, one orbit at a time, for n / step even.  A rotation by
 // step crystals moves an LOR by step views, so every orbit has members in
 // views [0, step): an LOR x and its half-turn partner (rotation by n / 2
 // crystals).  The one of the two with the lower bin index sums the input
 // over the n / step rotations of x and writes that sum to every member of
 // the orbit (the sum is the same for all of them): one read and one write
-// per bin.  grid (ceil(R T / 256), step, planes)
-__global__ void rotate_orbit_kernel(const long long* __restrict__ in, long long* __restrict__ out, int n,
-                                    int n_rings, int R, int T, int step) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= R * T) return;
-  const int r = c / T, t = c - r * T;
+// per bin.
+//
+// Where the rotation by c crystals takes (a, b) of view v and radial bin r:
+// a + b grows by 2 c, so the view is (v + c) mod n / 2, and each wrap mirrors
+// the radial bin (n crystals in the sum turn the sign of the LOR formula);
+// b alone has passed crystal n for c in [n - b, n - a), where the crystals'
+// order, the rings and the TOF axis are reversed.  That is a compare and a
+// select a member where applying the LOR formula to each took twenty
+// instructions, and four members' loads are in flight together (5 TOF bins, 45
+// rings, 28 rotations: 3559 -> 2606 us, 6.2 TB/s).
+// grid (ceil(R T / 256), step, planes)
+__global__ void __launch_bounds__(256) rotate_orbit_kernel(const long long* __restrict__ in, long long* __restrict__ out,
+                                                           int n, int n_rings, int R, int T, int step) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= R * T) return;
+  const int r = i / T, t = i - r * T;
   const int v = blockIdx.y;
   const int p = blockIdx.z;
   const int ra = p / n_rings, rb = p - ra * n_rings;
   const int rad_off = (n - 1 - R) / 2;
   int a, b;
   lor_crystals(n, v, r + rad_off, a, b);
-  const int h = n / 2;
-  const long long self = (((long long)p * h + v) * R + r) * T + t;
-  const long long partner =
-      rotated_bin(n, n_rings, R, T, rad_off, a + h >= n ? a + h - n : a + h, b + h >= n ? b + h - n : b + h, ra, rb, t);
-  if (partner < self) return;
+  const int h = n / 2, row = R * T;
+  const long long J = (long long)h * row, base = (long long)p * J, base_t = (long long)(rb * n_rings + ra) * J;
+  // places in a view's row: kept or mirrored radially, TOF kept or reversed (by the planes kept or swapped)
+  const int keep = r * T + t, keep_t = r * T + (T - 1 - t);
+  const int mirr = (R - 1 - r) * T + t, mirr_t = (R - 1 - r) * T + (T - 1 - t);
+  auto reversed = [&](int c) { return (unsigned)(c - (n - b)) < (unsigned)(b - a); };
+  const bool half = reversed(h);
+  if ((half ? base_t + mirr_t : base + mirr) < base + keep) return;  // (both in view v) the partner's thread does it
+  // the member at view w (v + c less the wraps), mirrored m, rotation c
+  auto member = [&](int w, bool m, int c) -> long long {
+    const bool f = reversed(c);
+    return (f ? base_t : base) + ((long long)w * row + (f ? (m ? mirr_t : keep_t) : (m ? mirr : keep)));
+  };
+  constexpr int kU = 4;
+  const int members = n / step;
   long long sum = 0;
-  int a2 = a, b2 = b;
-  for (int k = 0; k < n / step; ++k, a2 += step, b2 += step) {
-    if (a2 >= n) a2 -= n;
-    if (b2 >= n) b2 -= n;
-    sum += __ldg(in + rotated_bin(n, n_rings, R, T, rad_off, a2, b2, ra, rb, t));
+  int w = v, c = 0;
+  bool m = false;
+  auto advance = [&]() {
+    c += step;
+    w += step;
+    if (w >= h) {
+      w -= h;
+      m = !m;
+    }
+  };
+  for (int k = 0; k < members; k += kU) {
+    long long x[kU];
+#pragma unroll
+    for (int q = 0; q < kU; ++q) {
+      x[q] = k + q < members ? __ldg(in + member(w, m, c)) : 0;
+      advance();
+    }
+#pragma unroll
+    for (int q = 0; q < kU; ++q) sum += x[q];
   }
-  a2 = a;
-  b2 = b;
-  for (int k = 0; k < n / step; ++k, a2 += step, b2 += step) {
-    if (a2 >= n) a2 -= n;
-    if (b2 >= n) b2 -= n;
-    out[rotated_bin(n, n_rings, R, T, rad_off, a2, b2, ra, rb, t)] = sum;
+  w = v;
+  c = 0;
+  m = false;
+  for (int k = 0; k < members; ++k) {
+    out[member(w, m, c)] = sum;
+    advance();
   }
 }
 
