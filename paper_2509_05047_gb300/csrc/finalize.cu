@@ -127,15 +127,16 @@ __device__ __forceinline__ float i64_to_f32(long long v) {
   return __int_as_float((int)(((unsigned)(e + 127) << 23) | ((unsigned)m & 0x7fffffu)));
 }
 
-// float -> double (exact)
+// float -> double (exact), in 32-bit words
 __device__ __forceinline__ double f32_to_f64(float f) {
   const unsigned b = (unsigned)__float_as_int(f);
-  const unsigned ef = (b >> 23) & 0xffu;
-  if ((b & 0x7fffffffu) == 0) return (b >> 31) ? -0.0 : 0.0;
-  if (ef == 0 || ef == 0xffu) return hw_f32_to_f64(f);
-  return __longlong_as_double(((unsigned long long)(b >> 31) << 63) |
-                              ((unsigned long long)(ef - 127 + 1023) << 52) |
-                              ((unsigned long long)(b & 0x7fffffu) << 29));
+  unsigned hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20)), lo = b << 29;
+  if (((b >> 23) & 0xffu) - 1u >= 254u) {
+    if ((b << 1) != 0u) return hw_f32_to_f64(f);
+    hi = b;  // zero
+    lo = 0u;
+  }
+  return __hiloint2double((int)hi, (int)lo);
 }
 
 // double -> float (RNE) from the two 32-bit halves: the 23 kept mantissa
@@ -533,20 +534,20 @@ __device__ __forceinline__ double axial_epilogue(float y, long long qa, double f
   return use_sens ? mul_f32_f64(y, fs) : f32_to_f64(y);
 }
 
-// The same epilogue on the FP64 hardware: y widened (exact) and multiplied by
-// correctly rounded FP64 instructions, so the same bits as axial_epilogue.
-// GB300's FP64 pipe retires about 2 operations per clock per SM; the axial
+// The same epilogue with correctly rounded FP64 multiplies, so the same bits as
+// axial_epilogue; y is widened in integer words, which leaves the FP64 pipe
+// (about 2 operations per clock per SM) the products alone.  The direct axial
 // pass sends one output of each 2-output step here and the other through the
 // integer-pipe product, which splits the epilogue between the two pipes.
 template <bool kDivide, bool kNorm>
 __device__ __forceinline__ double axial_epilogue_fp64(float y, long long qa, double fr, double fs, bool use_sens,
                                                       float cf) {
-  if (kDivide) return (double)(qa != 0 ? y / (i64_to_f32(qa) * cf) : 0.0f);
+  if (kDivide) return f32_to_f64(qa != 0 ? y / (i64_to_f32(qa) * cf) : 0.0f);
   if (kNorm) {
-    const double x = (double)y * fr;
+    const double x = f32_to_f64(y) * fr;
     return use_sens ? x * fs : x;
   }
-  return use_sens ? (double)y * fs : (double)y;
+  return use_sens ? f32_to_f64(y) * fs : f32_to_f64(y);
 }
 
 // One axial column of an instantiated radius KT: the sliding window of slide
@@ -653,11 +654,32 @@ constexpr int kAxialMinCtas = KT >= 0 && KT <= 8 ? (kNorm ? 4 : 6) : 1;
 // the axial pass treats every bin alike) over the L planes of one segment:
 // one thread issues L row copies (cp.async.bulk.tensor, 1 KB each) into
 // shared memory at once, in groups of kTmaRows rows that complete on their
-// own mbarrier, and every thread slides down its column in shared memory,
+// own mbarrier, and every thread slides down its columns in shared memory,
 // waiting for a group only when its first row is needed.  Outputs, factors
 // and arithmetic are those of axial_column (bit-identical results).
+//
+// A thread has two neighbouring columns (J is a multiple of 4, so a pair never
+// straddles a plane's end): packed FMAs do both, rows are 8-byte loads and
+// estimates 16-byte stores.  Shared memory, not registers, limits the tiles on an
+// SM, so half the threads cost nothing.  Per block of 8 outputs it reads the
+// 8 + 2 KT rows from shared memory again instead of moving a register window
+// (8 moves an output at radius 8), at offsets from a table of reflected rows made
+// once a CTA.  The block's factors are loaded before its FMA chains, and the
+// products take the FP64 pipe alone (one output in 8 on the integer pipes: 1-4 %
+// slower).
+// With one column a thread and a register window the pass took 817 us on 448 x
+// 45 without TOF, radius 8 (4.1 GB), now 677 us (6.0 TB/s); the whole finalize
+// at 9 TOF bins 13.10 -> 11.14 ms, without TOF with a normalisation and radius 20
+// 4.74 -> 3.66 ms.
 // grid (ceil(J / 256), segments); shared memory: the launch's longest segment, in KB.
 // ---------------------------------------------------------------------------
+constexpr int kTileNb = 8;            // outputs of a column per block
+constexpr int kTileThreads = 768;     // resident threads per SM asked of the compiler: 6 tiles of 256 bins, 80 registers
+constexpr int kMaxWindow = 24;        // the largest instantiated radius
+// the axial weights, each twice (both columns of a pair), tap 0 to the centre
+struct PairWeights {
+  float2 g[kMaxWindow + 1];
+};
 constexpr int kTmaRows = 8;           // rows per mbarrier group
 constexpr int kTmaMaxRings = 96;      // tiles of at most 96 rows (96 KB of shared memory)
 constexpr int kTmaShortRows = 36;     // segments up to 36 planes: 6 CTAs of 36 KB tiles per SM
@@ -701,13 +723,15 @@ __device__ __forceinline__ void tma_row(float* dst, const CUtensorMap* map, int 
 // kFault (an instantiation for tests of the timeout path only): no copies are
 // issued for a tile's first row group, whose wait runs out after
 // kTmaFaultSpins polls; the other groups' copies run and are waited for.
-// TW: the tile's width in bins, which is also the CTA's thread count.
+// TW: the tile's width in bins, twice the CTA's thread count.
 template <int KT, bool kDivide, bool kNorm, bool kFault = false, int TW = kSmoothThreads>
-__global__ void __launch_bounds__(TW, (kAxialMinCtas<KT, kNorm> * kSmoothThreads / TW))
-    smooth_axial_tma_kernel(const __grid_constant__ FinParams P, const __grid_constant__ CUtensorMap map) {
+__global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
+    smooth_axial_tma_kernel(const __grid_constant__ FinParams P, const __grid_constant__ CUtensorMap map,
+                            const __grid_constant__ PairWeights W) {
   extern __shared__ __align__(128) float tile[];  // [L][TW]
   __shared__ __align__(8) unsigned long long bar[kTmaMaxRings / kTmaRows];
-  constexpr int NB = 2;
+  __shared__ __align__(16) int roff[kTmaMaxRings + 2 * kMaxWindow + 4];  // byte offset in the tile of row i - KT, reflected
+  constexpr int NB = kTileNb;
   const int nr = P.n_rings;
   const int seg = P.seg0 + (int)blockIdx.y;
   const int d = seg - (nr - 1);  // ring difference rb - ra
@@ -720,6 +744,8 @@ __global__ void __launch_bounds__(TW, (kAxialMinCtas<KT, kNorm> * kSmoothThreads
     for (int g = 0; g < ng; ++g) mbar_init(&bar[g], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  for (int i = threadIdx.x; i < (L + NB - 1) / NB * NB + 2 * KT; i += TW / 2)
+    roff[i] = reflect(i - KT, L) * (TW * (int)sizeof(float));
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int g = 0; g < ng; ++g) {
@@ -751,9 +777,9 @@ __global__ void __launch_bounds__(TW, (kAxialMinCtas<KT, kNorm> * kSmoothThreads
       }
     }
   };
-  const long long x = x0 + (long long)threadIdx.x;
+  const long long x = x0 + 2LL * threadIdx.x;  // the pair x, x + 1 (J is even)
   if (x >= J) {
-    // a column past the plane's end (zero-filled by the copy): no output, but
+    // columns past the plane's end (zero-filled by the copy): no output, but
     // the CTA's copies complete before any of its threads may end the CTA
     if (!need(L - 1)) give_up();
     return;
@@ -762,77 +788,87 @@ __global__ void __launch_bounds__(TW, (kAxialMinCtas<KT, kNorm> * kSmoothThreads
   const long long bin_step = (long long)(nr + 1) * J;  // next plane of the segment
   const long long lors = (long long)P.V * P.R;
   const long long lor0 = p0 * lors + fdiv((unsigned)x, P.magic_T);  // x T < 2^32 (host check)
+  const int lor1 = (int)(fdiv((unsigned)x + 1u, P.magic_T) - fdiv((unsigned)x, P.magic_T));  // 0, or 1 in the next LOR
   const long long lor_step = (long long)(nr + 1) * lors;
 #if PSC_DEBUG
-  if (dbg_idx(P.dbg, kSiteFinColumn, bin0 + (L - 1) * bin_step, P.n_bins) != bin0 + (L - 1) * bin_step ||
-      dbg_idx(P.dbg, kSiteFinLor, lor0 + (L - 1) * lor_step, P.n_bins / P.T) != lor0 + (L - 1) * lor_step) {
+  const long long bin_end = bin0 + 1 + (L - 1) * bin_step, lor_end = lor0 + lor1 + (L - 1) * lor_step;
+  if (dbg_idx(P.dbg, kSiteFinColumn, bin_end, P.n_bins) != bin_end ||
+      dbg_idx(P.dbg, kSiteFinLor, lor_end, P.n_bins / P.T) != lor_end) {
     if (!need(L - 1)) give_up();
     return;
   }
 #endif
-  const float* col = tile + threadIdx.x;  // row k at col[k * TW]
-  const Weights& g = P.g[2];
-  float w[2 * KT + NB];
-  if (L >= KT) {
-    if (KT > 0 && !need(KT - 1)) return give_up();
-#pragma unroll
-    for (int r = 0; r < KT; ++r) {  // row r, and row -1 - r reflected onto it
-      const float v = col[r * TW];
-      w[KT + r] = v;
-      w[KT - 1 - r] = v;
-    }
-  } else {
-    if (!need(L - 1)) return give_up();
-#pragma unroll
-    for (int j = 0; j < 2 * KT; ++j) w[j] = col[reflect(j - KT, L) * TW];
-  }
+  const char* col = reinterpret_cast<const char*>(tile) + threadIdx.x * sizeof(float2);
   const bool use_sens = !P.sens_first && P.sens;
   const float cf = (float)P.c;
-  const long long step2 = NB * bin_step;
   double* dst = P.out + bin0;
+  const bool wide = ((uintptr_t)P.out & 15) == 0;  // bin0 is even: 16-byte stores
   const long long* ap = P.acc + bin0;
   const long long rs = P.norm_per_lor ? lor_step : bin_step, ss = P.sens_per_lor ? lor_step : bin_step;
+  const int r1 = P.norm_per_lor ? lor1 : 1, s1 = P.sens_per_lor ? lor1 : 1;  // the second column's factor
   const double* rp = kNorm ? P.rnorm + (P.norm_per_lor ? lor0 : bin0) : nullptr;
   const double* sp = use_sens ? P.sens + (P.sens_per_lor ? lor0 : bin0) : nullptr;
   for (int o0 = 0; o0 < L; o0 += NB) {
-    if (!need(min(o0 + KT + 1, L - 1))) return give_up();
-    const int ra = o0 + KT < L ? o0 + KT : reflect(o0 + KT, L);
-    const int rb = o0 + KT + 1 < L ? o0 + KT + 1 : reflect(o0 + KT + 1, L);
-    w[2 * KT] = col[ra * TW];
-    w[2 * KT + 1] = col[rb * TW];
-    float s0 = 0.0f, s1 = 0.0f;
+    const int rows = min(NB, L - o0);
+    if (!need(min(o0 + NB - 1 + KT, L - 1))) return give_up();
+    // the block's factors, on their way during the FMA chains
+    double fs[NB][2];
+    if (!kDivide && use_sens) {
 #pragma unroll
-    for (int j = 0; j <= 2 * KT; ++j) {
-      s0 = fmaf(g[j], w[j], s0);
-      s1 = fmaf(g[j], w[j + 1], s1);
+      for (int q = 0; q < NB; ++q)
+        if (q < rows) {
+          fs[q][0] = __ldg(sp + q * ss);
+          fs[q][1] = __ldg(sp + q * ss + s1);
+        }
+      sp += NB * ss;
     }
-    const bool two = o0 + 1 < L;
-    long long qa0 = 0, qa1 = 0;
-    double fr0 = 1.0, fr1 = 1.0, fs0 = 1.0, fs1 = 1.0;
-    if (kDivide) {
-      qa0 = __ldg(ap);
-      if (two) qa1 = __ldg(ap + bin_step);
-      ap += step2;
-    } else {
+    float2 y[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) y[q] = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int j0 = 0; j0 < NB + 2 * KT; j0 += 4) {
+      const int4 ro = *reinterpret_cast<const int4*>(roff + o0 + j0);
+      const int at[4] = {ro.x, ro.y, ro.z, ro.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = j0 + u;
+        if (j >= NB + 2 * KT) break;
+        const float2 v = *reinterpret_cast<const float2*>(col + at[u]);
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+          const int k = j - q;  // tap of output o0 + q
+          if (k >= 0 && k <= 2 * KT) y[q] = __ffma2_rn(W.g[k <= KT ? k : 2 * KT - k], v, y[q]);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      if (q >= rows) break;
+      long long qa0 = 0, qa1 = 0;
+      double fr0 = 1.0, fr1 = 1.0;
+      if (kDivide) {
+        qa0 = __ldg(ap + q * bin_step);
+        qa1 = __ldg(ap + q * bin_step + 1);
+      }
       if (kNorm) {
-        fr0 = __ldg(rp);
-        if (two) fr1 = __ldg(rp + rs);
-        rp += NB * rs;
+        fr0 = __ldg(rp + q * rs);
+        fr1 = __ldg(rp + q * rs + r1);
       }
-      if (use_sens) {
-        fs0 = __ldg(sp);
-        if (two) fs1 = __ldg(sp + ss);
-        sp += NB * ss;
+      const double e0 = axial_epilogue_fp64<kDivide, kNorm>(y[q].x, qa0, fr0, fs[q][0], use_sens, cf);
+      const double e1 = axial_epilogue_fp64<kDivide, kNorm>(y[q].y, qa1, fr1, fs[q][1], use_sens, cf);
+      double* o = dst + q * bin_step;
+      if (wide) {
+        *reinterpret_cast<double2*>(o) = make_double2(e0, e1);
+      } else {
+        o[0] = e0;
+        o[1] = e1;
       }
     }
-    dst[0] = axial_epilogue<kDivide, kNorm>(s0, qa0, fr0, fs0, use_sens, cf);
-    if (two) dst[bin_step] = axial_epilogue_fp64<kDivide, kNorm>(s1, qa1, fr1, fs1, use_sens, cf);
-    dst += step2;
-#pragma unroll
-    for (int j = 0; j < 2 * KT; ++j) w[j] = w[NB + j];
+    dst += NB * bin_step;
+    if (kDivide) ap += NB * bin_step;
+    if (kNorm) rp += NB * rs;
   }
 }
-
 
 template <int KT, bool kDivide, bool kNorm>
 __global__ void __launch_bounds__(kSmoothThreads, (kAxialMinCtas<KT, kNorm>)) smooth_axial_kernel(const __grid_constant__ FinParams P) {
@@ -1059,7 +1095,9 @@ static cudaError_t run_axial_tma(const FinParams& p, const CUtensorMap& map, dim
   auto k = smooth_axial_tma_kernel<KT, kDivide, kNorm, kFault, TW>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<grid, TW, smem, s>>>(p, map);
+  PairWeights w = {};
+  for (int j = 0; j <= KT; ++j) w.g[j] = make_float2(p.g[2][j], p.g[2][j]);
+  k<<<grid, TW / 2, smem, s>>>(p, map, w);
   return cudaGetLastError();
 }
 
