@@ -118,13 +118,15 @@ __device__ __forceinline__ double i64_to_f64(long long v) {
   return __longlong_as_double(((unsigned long long)(e + 1023) << 52) | (m & kMant52));
 }
 
-// non-negative int64 -> float (RNE)
+// non-negative int64 -> float (RNE): the top 32 significant bits in a word, the
+// bits below as its lowest bit (a sticky bit, 8 places below the rounding), one
+// 32-bit conversion and an exact scaling by a power of two
 __device__ __forceinline__ float i64_to_f32(long long v) {
-  const unsigned long long u = (unsigned long long)v;
-  if (u == 0) return 0.0f;
-  int e = msb64(u);
-  unsigned long long m = e <= 23 ? u << (23 - e) : rne_shift(u, e - 23, false, 24, e);
-  return __int_as_float((int)(((unsigned)(e + 127) << 23) | ((unsigned)m & 0x7fffffu)));
+  const unsigned hi = (unsigned)((unsigned long long)v >> 32), lo = (unsigned)v;
+  const unsigned top = hi ? hi : lo, next = hi ? lo : 0u;
+  const int s = __clz((int)top);  // 32 for zero
+  const unsigned w = __funnelshift_lc(next, top, s) | (__funnelshift_lc(0u, next, s) != 0u ? 1u : 0u);
+  return __uint2float_rn(w) * __int_as_float(((hi ? 159 : 127) - s) << 23);
 }
 
 // float -> double (exact), in 32-bit words
@@ -383,6 +385,12 @@ __global__ void __launch_bounds__(256) finalize_plain_kernel(const __grid_consta
 // ---------------------------------------------------------------------------
 using Weights = float[2 * kMaxSmoothRadius + 1];
 
+constexpr int kMaxWindow = 24;        // the largest instantiated radius
+// an axis's weights, each twice (a pair of columns shares them), tap 0 to the centre: they are symmetric
+struct PairWeights {
+  float2 g[kMaxWindow + 1];
+};
+
 template <int KT, int NBS, class In, class Cvt, class Store>
 __device__ __forceinline__ void slide(const In* __restrict__ src, long long stride, int n, const Weights& g,
                                       Cvt cvt, Store store) {
@@ -489,6 +497,127 @@ __global__ void __launch_bounds__(kSmoothThreads) smooth_radial_kernel(const __g
       if (r0 + q < R) dst[(r0 + q) * T] = y[q];
   };
   slide_any<KT>(P.acc + base, T, R, P.K[0], P.g[0], cvt, store);
+}
+
+// ---------------------------------------------------------------------------
+// pass A for short TOF axes: whole radial lines staged in shared memory.
+// A column's neighbours along rad lie T bins apart, so with few TOF bins the
+// kernel above touches a new sector per thread and load, and a plane has few
+// columns: without TOF it moved 2.4 GB in 1.77 ms.  Here a CTA takes G pairs of
+// lines of a plane: its threads load them bin by bin (up to 16 loads each in
+// flight), convert every bin once and store it, with the rows that the line's
+// edges reflect, in shared memory, a pair's two lines side by side.  A thread then
+// computes 8 consecutive radial outputs of one TOF bin of both lines with
+// packed FMAs from 8 + 2 KT rows, and the outputs go back through shared
+// memory to coalesced stores.  Same conversion and same FMA chains.
+// Rows lie in blocks of 8 rows of T values, block pitch S = 8 T + pad, chosen by
+// the host so that a half-warp's lanes (block, tof) read different banks.
+// Radius 8, 448 x 45 scanner, radial pass: 1 TOF bin 1798 -> 572 us (with one
+// line a thread 896), 3 TOF bins 2088 -> 1737 us, 5 TOF bins 2523 -> 2889 us:
+// taken up to kLineMaxT TOF bins.
+// grid (ceil(V / (2 G)), planes)
+// ---------------------------------------------------------------------------
+constexpr int kLineMaxT = 4;
+constexpr int kLineThreads = 512, kLineCtas = 2;
+struct LineStage {
+  int G;            // pairs of lines per CTA
+  int RB;           // output blocks of 8 rows a line
+  int S;            // pitch of a block of 8 rows
+  int LP;           // pitch of a line, halo included
+  unsigned magic_line, magic_block, magic_items;  // exact division by R T, 8 T and RB T
+};
+
+template <int KT>
+__global__ void __launch_bounds__(kLineThreads, kLineCtas)
+    smooth_radial_lines_kernel(const __grid_constant__ FinParams P, const __grid_constant__ LineStage H,
+                               const __grid_constant__ PairWeights W) {
+  extern __shared__ __align__(16) float2 rows[];
+  constexpr int NB = 8;
+  const int R = P.R, T = P.T, RT = R * T, T8 = 8 * T;
+  const int v0 = blockIdx.x * 2 * H.G, lines = min(2 * H.G, P.V - v0), n = (lines + 1) / 2 * RT;
+  const long long line0 = plane_at(P, blockIdx.y) * P.V + v0, base = line0 * RT, lor0 = line0 * R;
+  const float cf = (float)P.c;
+  const bool with_sens = P.sens_first && P.sens;
+  const int step = blockDim.x;
+  long long raw[NB][2];
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {  // the launch has at least n / 8 threads
+    const int e = threadIdx.x + i * step, g = (int)fdiv((unsigned)e, H.magic_line);
+    raw[i][0] = raw[i][1] = 0;
+    if (e < n) {
+      const long long bin = base + e + (long long)g * RT;  // line 2 g, and RT further on its partner
+      raw[i][0] = __ldg(P.acc + dbg_idx(P.dbg, kSiteFinBin, bin, P.n_bins));
+      if (2 * g + 1 < lines) raw[i][1] = __ldg(P.acc + dbg_idx(P.dbg, kSiteFinBin, bin + RT, P.n_bins));
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int e = threadIdx.x + i * step;
+    if (e >= n) break;
+    const int g = (int)fdiv((unsigned)e, H.magic_line), at = e - g * RT;  // at: rad T + tof
+    float2 x = make_float2(i64_to_f32(raw[i][0]) * cf, i64_to_f32(raw[i][1]) * cf);
+    if (with_sens || P.norm) {
+      const long long bin = base + e + (long long)g * RT;
+      const long long lor = lor0 + 2LL * g * R + fdiv((unsigned)at, P.magic_T);
+      const int two = 2 * g + 1 < lines;
+#if PSC_DEBUG
+      if (dbg_idx(P.dbg, kSiteFinLor, lor + two * R, P.n_bins / T) != lor + two * R) continue;
+#endif
+      if (with_sens) {
+        x.x *= factor(P.sens32, P.sens, P.sens_per_lor ? lor : bin);
+        x.y *= factor(P.sens32, P.sens, P.sens_per_lor ? lor + two * R : bin + two * RT);
+      }
+      if (P.norm) {
+        x.x *= factor(P.norm32, P.norm, P.norm_per_lor ? lor : bin);
+        x.y *= factor(P.norm32, P.norm, P.norm_per_lor ? lor + two * R : bin + two * RT);
+      }
+    }
+    float2* line = rows + g * H.LP;
+    auto place = [&](int k) {  // k: row T + tof, rows counted from the halo's first
+      return k + (int)fdiv((unsigned)k, H.magic_block) * (H.S - T8);
+    };
+    line[place(at + KT * T)] = x;
+    if (at < KT * T || at >= RT - KT * T) {  // rows that an edge reflects
+      const int r = (int)fdiv((unsigned)at, P.magic_T), t = at - r * T;
+      if (r < KT) line[place((KT - 1 - r) * T + t)] = x;
+      if (r >= R - KT) line[place((2 * R - 1 - r + KT) * T + t)] = x;
+    }
+  }
+  __syncthreads();
+  const int items = H.RB * T, gi = (int)fdiv(threadIdx.x, H.magic_items), item = threadIdx.x - gi * items;
+  const bool mine = 2 * gi < lines && gi < H.G;
+  const int b = (int)fdiv((unsigned)item, P.magic_T), t = item - b * T;
+  float2* own = rows + gi * H.LP + b * H.S + t;  // rows 8 b and on: the outputs', and (from the halo's first) the inputs'
+  float2 y[NB];
+#pragma unroll
+  for (int q = 0; q < NB; ++q) y[q] = make_float2(0.0f, 0.0f);
+  if (mine) {
+#pragma unroll
+    for (int j = 0; j < NB + 2 * KT; ++j) {
+      const float2 x = own[(j >> 3) * H.S + (j & 7) * T];
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        const int k = j - q;
+        if (k >= 0 && k <= 2 * KT) y[q] = __ffma2_rn(W.g[k <= KT ? k : 2 * KT - k], x, y[q]);
+      }
+    }
+  }
+  __syncthreads();
+  if (mine) {
+#pragma unroll
+    for (int q = 0; q < NB; ++q) own[q * T] = y[q];  // rows past R - 1 land in the line's unused places
+  }
+  __syncthreads();
+  float* dst = reinterpret_cast<float*>(P.out) + base;
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int e = threadIdx.x + i * step;
+    if (e >= n) break;
+    const int g = (int)fdiv((unsigned)e, H.magic_line), at = e - g * RT;
+    const float2 o = rows[g * H.LP + at + (int)fdiv((unsigned)at, H.magic_block) * (H.S - T8)];
+    dst[e + (long long)g * RT] = o.x;
+    if (2 * g + 1 < lines) dst[e + (long long)g * RT + RT] = o.y;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -675,11 +804,6 @@ constexpr int kAxialMinCtas = KT >= 0 && KT <= 8 ? (kNorm ? 4 : 6) : 1;
 // ---------------------------------------------------------------------------
 constexpr int kTileNb = 8;            // outputs of a column per block
 constexpr int kTileThreads = 768;     // resident threads per SM asked of the compiler: 6 tiles of 256 bins, 80 registers
-constexpr int kMaxWindow = 24;        // the largest instantiated radius
-// the axial weights, each twice (both columns of a pair), tap 0 to the centre
-struct PairWeights {
-  float2 g[kMaxWindow + 1];
-};
 constexpr int kTmaRows = 8;           // rows per mbarrier group
 constexpr int kTmaMaxRings = 96;      // tiles of at most 96 rows (96 KB of shared memory)
 constexpr int kTmaShortRows = 36;     // segments up to 36 planes: 6 CTAs of 36 KB tiles per SM
@@ -1040,12 +1164,80 @@ int finalize_planes(const FinParams& p) {
   return n;
 }
 
+template <int KT>
+static PairWeights pair_weights(const Weights& g) {
+  PairWeights w = {};
+  for (int j = 0; j <= KT; ++j) w.g[j] = make_float2(g[j], g[j]);
+  return w;
+}
+
+template <int I = 0, class F>
+static cudaError_t for_window_radius(int kt, F&& f) {
+  constexpr int n = (int)(sizeof(kWindowRadii) / sizeof(kWindowRadii[0]));
+  if constexpr (I == n) {
+    return cudaErrorInvalidValue;
+  } else {
+    if (kt == kWindowRadii[I]) return f(std::integral_constant<int, kWindowRadii[I]>{});
+    return for_window_radius<I + 1>(kt, f);
+  }
+}
+
+// The staged radial pass takes short TOF axes whose lines fit a CTA: an
+// instantiated radius no larger than the line (one reflection), at most 512
+// threads of 8 x 2 outputs, 100 KB of shared memory, and exact divisions by
+// multiply-high.
+static bool line_stage(const FinParams& p, LineStage* h) {
+  const int KT = p.KT[0], R = p.R, T = p.T;
+  if (KT < 0 || R < KT || T > kLineMaxT) return false;
+  const int RB = (R + 7) / 8, items = RB * T;
+  if (items > kLineThreads) return false;
+  h->RB = RB;
+  h->G = std::min((p.V + 1) / 2, std::max(1, 256 / items));
+  // lanes run over tof, then blocks, and read 8 bytes each, 16 lanes at a time: up to
+  // 7 places of padding a block, the fewest lanes on one bank pair
+  int best = 1 << 30;
+  for (int pad = 0; pad < 8; ++pad) {
+    int worst = 0, hits[2][16] = {};
+    for (int lane = 0; lane < 32; ++lane)
+      worst = std::max(worst, ++hits[lane / 16][(lane / T * (8 * T + pad) + lane % T) & 15]);
+    if (worst < best) {
+      best = worst;
+      h->S = 8 * T + pad;
+    }
+  }
+  h->LP = (R + 2 * KT + 7 + 7) / 8 * h->S;  // the last block's rows reach 8 RB - 1 + 2 KT <= R + 6 + 2 KT
+  const long long n = (long long)h->G * R * T + kLineThreads * 8;
+  if ((size_t)h->G * h->LP * sizeof(float2) > 100 * 1024) return false;
+  if (n * R * T >= (1LL << 32) || ((long long)R + 2 * KT) * T * 8 * T >= (1LL << 32) || (kLineThreads + 31LL) * items >= (1LL << 32))
+    return false;
+  auto magic = [](int d) { return d == 1 ? 0u : (unsigned)(((1ULL << 32) + d - 1) / d); };
+  h->magic_line = magic(R * T);
+  h->magic_block = magic(8 * T);
+  h->magic_items = magic(items);
+  return true;
+}
+
 cudaError_t launch_smooth_front(const FinParams& p, cudaStream_t s) {
   cudaError_t e;
   const unsigned planes = (unsigned)finalize_planes(p);
   const long long I = (long long)p.R * p.T;
-  if ((e = dispatch_kt<RadialL>(p.KT[0], p, dim3(smooth_blocks((long long)p.V * p.T), planes), s)) != cudaSuccess)
-    return e;
+  LineStage h;
+  if (line_stage(p, &h)) {
+    const dim3 grid((unsigned)((p.V + 2 * h.G - 1) / (2 * h.G)), planes);
+    const int threads = (h.G * h.RB * p.T + 31) / 32 * 32;
+    const size_t smem = (size_t)h.G * h.LP * sizeof(float2);
+    e = for_window_radius(p.KT[0], [&](auto kt) -> cudaError_t {
+      constexpr int KT = decltype(kt)::value;
+      const cudaError_t a = cudaFuncSetAttribute(smooth_radial_lines_kernel<KT>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (a != cudaSuccess) return a;
+      smooth_radial_lines_kernel<KT><<<grid, threads, smem, s>>>(p, h, pair_weights<KT>(p.g[0]));
+      return cudaGetLastError();
+    });
+  } else {
+    e = dispatch_kt<RadialL>(p.KT[0], p, dim3(smooth_blocks((long long)p.V * p.T), planes), s);
+  }
+  if (e != cudaSuccess) return e;
   return dispatch_kt<ViewL>(p.KT[1], p, dim3(smooth_blocks(I), planes), s);
 }
 
@@ -1095,21 +1287,8 @@ static cudaError_t run_axial_tma(const FinParams& p, const CUtensorMap& map, dim
   auto k = smooth_axial_tma_kernel<KT, kDivide, kNorm, kFault, TW>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  PairWeights w = {};
-  for (int j = 0; j <= KT; ++j) w.g[j] = make_float2(p.g[2][j], p.g[2][j]);
-  k<<<grid, TW / 2, smem, s>>>(p, map, w);
+  k<<<grid, TW / 2, smem, s>>>(p, map, pair_weights<KT>(p.g[2]));
   return cudaGetLastError();
-}
-
-template <int I = 0, class F>
-static cudaError_t for_window_radius(int kt, F&& f) {
-  constexpr int n = (int)(sizeof(kWindowRadii) / sizeof(kWindowRadii[0]));
-  if constexpr (I == n) {
-    return cudaErrorInvalidValue;
-  } else {
-    if (kt == kWindowRadii[I]) return f(std::integral_constant<int, kWindowRadii[I]>{});
-    return for_window_radius<I + 1>(kt, f);
-  }
 }
 
 cudaError_t launch_smooth_axial(const FinParams& p, int lo, int hi, cudaStream_t s) {
