@@ -6,6 +6,7 @@
 // validate their arguments, never throw across the ABI, and enqueue kernels
 // on the caller's stream.
 #include <cerrno>
+#include <cfloat>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -288,55 +289,6 @@ const char* kind_name(int k) {
 #define GET(T, var, id, kind)                                                     \
   auto var = get<T>(ctx, id, kind);                                               \
   if (!var) return fail(PSC_ENOTFOUND, "no %s with id %d", kind_name(kind), (int)(id))
-
-// ---------------------------------------------------------------------------
-// Vose's alias method (Vose 1991) in FP64 with a fixed work-list order:
-// scaled weights n * a_i / sum, indices pushed in ascending order onto a
-// "small" (< 1) or "large" stack, pairs popped from the tops; leftovers get
-// probability 1.
-// ---------------------------------------------------------------------------
-int build_alias(const float* a, long long n, std::vector<double>& prob, std::vector<int32_t>& alias) {
-  double sum = 0.0;
-  for (long long i = 0; i < n; ++i) {
-    const double v = (double)a[i];
-    if (!(v >= 0.0) || !std::isfinite(v)) return fail(PSC_EINVAL, "activity[%lld] is negative or not finite", i);
-    sum += v;
-  }
-  if (!(sum > 0.0) || !std::isfinite(sum)) return fail(PSC_EINVAL, "activity has no positive finite sum");
-  prob.assign((size_t)n, 0.0);
-  alias.assign((size_t)n, 0);
-  std::vector<double> p((size_t)n);
-  std::vector<int32_t> small, large;
-  small.reserve((size_t)n);
-  large.reserve((size_t)n);
-  for (long long i = 0; i < n; ++i) {
-    p[i] = ((double)a[i] * (double)n) / sum;
-    (p[i] < 1.0 ? small : large).push_back((int32_t)i);
-  }
-  while (!small.empty() && !large.empty()) {
-    const int32_t s = small.back();
-    small.pop_back();
-    const int32_t l = large.back();
-    large.pop_back();
-    prob[s] = p[s];
-    alias[s] = l;
-    p[l] = (p[l] + p[s]) - 1.0;
-    (p[l] < 1.0 ? small : large).push_back(l);
-  }
-  while (!large.empty()) {
-    const int32_t l = large.back();
-    large.pop_back();
-    prob[l] = 1.0;
-    alias[l] = l;
-  }
-  while (!small.empty()) {
-    const int32_t s = small.back();
-    small.pop_back();
-    prob[s] = 1.0;
-    alias[s] = s;
-  }
-  return PSC_OK;
-}
 
 float round_up_f32(double v) {
   float f = (float)v;
@@ -669,22 +621,84 @@ int psc_load_materials(psc_ctx* ctx, const psc_materials_desc* d, int32_t* id) {
 // k = x >> 9, satisfies u < p exactly when k < ceil((p 2^24 - 1) / 2), so the
 // kernel decides with one integer compare what the FP64 comparison decides.
 static uint32_t alias_threshold(double p) {
-  const double t = std::ceil((std::ldexp(p, 24) - 1.0) / 2.0);
+  const double t = (p * 16777216.0 - 1.0) / 2.0;
   if (!(t > 0.0)) return 0u;
-  return t >= 8388608.0 ? 8388608u : (uint32_t)t;
+  if (t >= 8388608.0) return 8388608u;
+  const uint32_t k = (uint32_t)t;
+  return k + ((double)k < t);
 }
 
 }  // extern "C"
 
 namespace psc {
 
+// ---------------------------------------------------------------------------
+// Vose's alias method (Vose 1991) in FP64 with a fixed work-list order:
+// scaled weights n * a_i / sum, indices pushed in ascending order onto a
+// "small" (< 1) or "large" stack, pairs popped from the tops; leftovers get
+// probability 1.
+//
+// A user who updates the activity waits for this on every iteration, so it is
+// one pass a step over flat arrays that are not cleared first: the two
+// stacks are filled without a branch (its outcome is the voxel's, not
+// predictable), the entry that a pair pushes back is the next one popped and
+// stays in registers with its weight, and thresholds are written as pairs are
+// made.
+// ---------------------------------------------------------------------------
 int alias_table(const float* activity, long long n_vox, std::vector<uint2>& tab) {
-  std::vector<double> prob;
-  std::vector<int32_t> alias;
-  int rc = build_alias(activity, n_vox, prob, alias);
-  if (rc) return rc;
-  tab.resize((size_t)n_vox);
-  for (long long i = 0; i < n_vox; ++i) tab[i] = make_uint2(alias_threshold(prob[i]), (uint32_t)alias[i]);
+  double sum = 0.0;
+  for (long long i = 0; i < n_vox; ++i) {
+    const float v = activity[i];
+    if (!(v >= 0.0f && v <= FLT_MAX)) return fail(PSC_EINVAL, "activity[%lld] is negative or not finite", i);
+    sum += (double)v;
+  }
+  if (!(sum > 0.0) || !std::isfinite(sum)) return fail(PSC_EINVAL, "activity has no positive finite sum");
+  const size_t n = (size_t)n_vox;
+  const std::unique_ptr<double[]> p(new double[n]);
+  const std::unique_ptr<int32_t[]> small(new int32_t[n]), large(new int32_t[n]);
+  for (size_t i = 0; i < n; ++i) p[i] = ((double)activity[i] * (double)n_vox) / sum;
+  size_t ns = 0, nl = 0;
+  for (size_t i = 0; i < n; ++i) {
+    small[ns] = large[nl] = (int32_t)i;
+    const bool below = p[i] < 1.0;
+    ns += below;
+    nl += !below;
+  }
+  tab.resize(n);
+  if (ns && nl) {
+    int32_t s = small[--ns], l = large[--nl];
+    double ps = p[s], pl = p[l];
+    for (;;) {
+      tab[s] = make_uint2(alias_threshold(ps), (uint32_t)l);
+      pl = (pl + ps) - 1.0;
+      if (pl < 1.0) {  // l is now the top of the small ones
+        if (!nl) {
+          small[ns++] = l;
+          break;
+        }
+        s = l;
+        ps = pl;
+        l = large[--nl];
+        pl = p[l];
+      } else {  // l stays the top of the large ones
+        if (!ns) {
+          large[nl++] = l;
+          break;
+        }
+        s = small[--ns];
+        ps = p[s];
+      }
+    }
+  }
+  const uint32_t one = alias_threshold(1.0);
+  while (nl) {
+    const int32_t l = large[--nl];
+    tab[l] = make_uint2(one, (uint32_t)l);
+  }
+  while (ns) {
+    const int32_t s = small[--ns];
+    tab[s] = make_uint2(one, (uint32_t)s);
+  }
   return PSC_OK;
 }
 
