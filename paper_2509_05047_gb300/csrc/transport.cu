@@ -460,7 +460,9 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
         // ---- emission (stream 0, words 0..6) ----
         // (the slot takes the work item's next history, if there is one)
         const unsigned off = sec == kEmit ? atomicAdd(&s_next, 1u) : ~0u;
-        if (off < s_len) {
+        const bool emitted = off < s_len;
+        float4 pos, dir;
+        if (emitted) {
           m = off << kMetaHistory;
           const uint4 b0 = block(0, 0), b1 = block(1, 0);
           const uint32_t w0 = b0.x, w1 = b0.y;
@@ -505,16 +507,24 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
           }
           setC(C_E0, g, ex, ey, ez, (uint32_t)v);
           setC(C_D0, g, dx, dy, dz, 0u);
-          s_pos[g] = make_float4(ex, ey, ez, 0.0f);
-          s_dir[g] = make_float4(dx, dy, dz, kEmitKeV);
-          s_kc[g] = make_uint2(0u, 0u);
-          s_meta[g] = flags | m;
+          s_pos[g] = pos = make_float4(ex, ey, ez, 0.0f);
+          s_dir[g] = dir = make_float4(dx, dy, dz, kEmitKeV);
+          m |= flags;
+          const uint4 b = block(0, (m >> 4) & 3u);
+          s_ring[g] = b;
+          kc = make_uint2(kKcBlock + 4u, 0u);
+          r0 = b.x;
+          r1 = b.y;
         }
 
-        // ---- one Woodcock step ----
-        if (sec == kStep) {
+        // ---- one Woodcock step (a new history takes its first one at once: a
+        // vote, a pass over the slots and a reload of its state fewer) ----
+        if (sec == kStep || emitted) {
           const uint32_t cnt = kc.y;
-          const float4 pos = s_pos[g], dir = s_dir[g];
+          if (!emitted) {
+            pos = s_pos[g];
+            dir = s_dir[g];
+          }
           const float e = dir.w;
           const float mu_max = interp_scalar(s_maj, ph.n_tab, ph.e0, e);
           bool moved = false;
@@ -526,7 +536,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
               reinterpret_cast<uint32_t*>(s_ring + g)[3] = r0;
               kc.x -= kKcBlock + 4u;
             }
-            s_kc[g].x = kc.x;
+            s_kc[g] = kc;
             set_section(kEscape);
           } else {
             const float px = pos.x, py = pos.y, pz = pos.z;
