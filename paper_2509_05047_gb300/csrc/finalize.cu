@@ -385,10 +385,10 @@ __global__ void __launch_bounds__(256) finalize_plain_kernel(const __grid_consta
 // ---------------------------------------------------------------------------
 using Weights = float[2 * kMaxSmoothRadius + 1];
 
-constexpr int kMaxWindow = 24;        // the largest instantiated radius
+constexpr int kWideRadius = 32;       // the axial tiles also take radii from 25 to this one
 // an axis's weights, each twice (a pair of columns shares them), tap 0 to the centre: they are symmetric
 struct PairWeights {
-  float2 g[kMaxWindow + 1];
+  float2 g[kWideRadius + 1];
 };
 
 template <int KT, int NBS, class In, class Cvt, class Store>
@@ -630,13 +630,13 @@ __global__ void __launch_bounds__(kSmoothThreads) smooth_view_kernel(const __gri
   const int I = P.R * P.T;
   const int i = blockIdx.x * kSmoothThreads + threadIdx.x;
   if (i >= I) return;
-  const long long base = plane_at(P, blockIdx.y) * P.V * I + i;
+  const long long plane = plane_at(P, blockIdx.y), base = plane * P.V * I + i;
 #if PSC_DEBUG
   if (dbg_idx(P.dbg, kSiteFinColumn, base + (long long)(P.V - 1) * I, P.n_bins) != base + (long long)(P.V - 1) * I)
     return;
 #endif
   const float* src = reinterpret_cast<const float*>(P.out) + base;
-  float* dst = P.scratch + base;
+  float* dst = P.scratch + plane * P.pitch + i;
   auto cvt = [](float x, int) { return x; };
   const int V = P.V;
   auto store = [&](int v0, const float (&y)[NB]) {
@@ -787,9 +787,8 @@ constexpr int kAxialMinCtas = KT >= 0 && KT <= 8 ? (kNorm ? 4 : 6) : 1;
 // waiting for a group only when its first row is needed.  Outputs, factors
 // and arithmetic are those of axial_column (bit-identical results).
 //
-// A thread has two neighbouring columns (J is a multiple of 4, so a pair never
-// straddles a plane's end): packed FMAs do both, rows are 8-byte loads and
-// estimates 16-byte stores.  Shared memory, not registers, limits the tiles on an
+// A thread has two neighbouring columns: packed FMAs do both, rows are 8-byte
+// loads and estimates 16-byte stores (8-byte ones where J is odd).  Shared memory, not registers, limits the tiles on an
 // SM, so half the threads cost nothing.  Per block of 8 outputs it reads the
 // 8 + 2 KT rows from shared memory again instead of moving a register window
 // (8 moves an output at radius 8), at offsets from a table of reflected rows made
@@ -854,7 +853,7 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
                             const __grid_constant__ PairWeights W) {
   extern __shared__ __align__(128) float tile[];  // [L][TW]
   __shared__ __align__(8) unsigned long long bar[kTmaMaxRings / kTmaRows];
-  __shared__ __align__(16) int roff[kTmaMaxRings + 2 * kMaxWindow + 4];  // byte offset in the tile of row i - KT, reflected
+  __shared__ __align__(16) int roff[kTmaMaxRings + 2 * kWideRadius + 4];  // byte offset in the tile of row i - KT, reflected
   constexpr int NB = kTileNb;
   const int nr = P.n_rings;
   const int seg = P.seg0 + (int)blockIdx.y;
@@ -901,7 +900,7 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
       }
     }
   };
-  const long long x = x0 + 2LL * threadIdx.x;  // the pair x, x + 1 (J is even)
+  const long long x = x0 + 2LL * threadIdx.x;  // the pair x, x + 1
   if (x >= J) {
     // columns past the plane's end (zero-filled by the copy): no output, but
     // the CTA's copies complete before any of its threads may end the CTA
@@ -912,24 +911,28 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
   const long long bin_step = (long long)(nr + 1) * J;  // next plane of the segment
   const long long lors = (long long)P.V * P.R;
   const long long lor0 = p0 * lors + fdiv((unsigned)x, P.magic_T);  // x T < 2^32 (host check)
-  const int lor1 = (int)(fdiv((unsigned)x + 1u, P.magic_T) - fdiv((unsigned)x, P.magic_T));  // 0, or 1 in the next LOR
+  const int two = x + 1 < J;  // the pair's second column (an odd plane's last bin has none)
+  const int lor1 = two ? (int)(fdiv((unsigned)x + 1u, P.magic_T) - fdiv((unsigned)x, P.magic_T)) : 0;  // 1: in the next LOR
   const long long lor_step = (long long)(nr + 1) * lors;
 #if PSC_DEBUG
-  const long long bin_end = bin0 + 1 + (L - 1) * bin_step, lor_end = lor0 + lor1 + (L - 1) * lor_step;
+  const long long bin_end = bin0 + two + (L - 1) * bin_step, lor_end = lor0 + lor1 + (L - 1) * lor_step;
   if (dbg_idx(P.dbg, kSiteFinColumn, bin_end, P.n_bins) != bin_end ||
       dbg_idx(P.dbg, kSiteFinLor, lor_end, P.n_bins / P.T) != lor_end) {
     if (!need(L - 1)) give_up();
     return;
   }
 #endif
+  // the wide window stands for radii from 25 on: taps beyond the radius are left out (a
+  // zero weight would spread an infinity further than the radius)
+  const int skip = KT == kWideRadius ? KT - P.K[2] : 0;
   const char* col = reinterpret_cast<const char*>(tile) + threadIdx.x * sizeof(float2);
   const bool use_sens = !P.sens_first && P.sens;
   const float cf = (float)P.c;
   double* dst = P.out + bin0;
-  const bool wide = ((uintptr_t)P.out & 15) == 0;  // bin0 is even: 16-byte stores
+  const bool wide = ((uintptr_t)P.out & 15) == 0 && J % 2 == 0;  // bin0 is even: 16-byte stores
   const long long* ap = P.acc + bin0;
   const long long rs = P.norm_per_lor ? lor_step : bin_step, ss = P.sens_per_lor ? lor_step : bin_step;
-  const int r1 = P.norm_per_lor ? lor1 : 1, s1 = P.sens_per_lor ? lor1 : 1;  // the second column's factor
+  const int r1 = P.norm_per_lor ? lor1 : two, s1 = P.sens_per_lor ? lor1 : two;  // the second column's factor
   const double* rp = kNorm ? P.rnorm + (P.norm_per_lor ? lor0 : bin0) : nullptr;
   const double* sp = use_sens ? P.sens + (P.sens_per_lor ? lor0 : bin0) : nullptr;
   for (int o0 = 0; o0 < L; o0 += NB) {
@@ -961,7 +964,9 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
           const int k = j - q;  // tap of output o0 + q
-          if (k >= 0 && k <= 2 * KT) y[q] = __ffma2_rn(W.g[k <= KT ? k : 2 * KT - k], v, y[q]);
+          if (k < 0 || k > 2 * KT) continue;
+          const int c = k <= KT ? k : 2 * KT - k;
+          if (KT < kWideRadius || c >= 8 || c >= skip) y[q] = __ffma2_rn(W.g[c], v, y[q]);
         }
       }
     }
@@ -972,7 +977,7 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
       double fr0 = 1.0, fr1 = 1.0;
       if (kDivide) {
         qa0 = __ldg(ap + q * bin_step);
-        qa1 = __ldg(ap + q * bin_step + 1);
+        qa1 = __ldg(ap + q * bin_step + two);
       }
       if (kNorm) {
         fr0 = __ldg(rp + q * rs);
@@ -985,7 +990,7 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
         *reinterpret_cast<double2*>(o) = make_double2(e0, e1);
       } else {
         o[0] = e0;
-        o[1] = e1;
+        if (two) o[1] = e1;
       }
     }
     dst += NB * bin_step;
@@ -1164,10 +1169,11 @@ int finalize_planes(const FinParams& p) {
   return n;
 }
 
+// weights centred on c in an array, for a window of radius KT >= c
 template <int KT>
-static PairWeights pair_weights(const Weights& g) {
+static PairWeights pair_weights(const Weights& g, int c = KT) {
   PairWeights w = {};
-  for (int j = 0; j <= KT; ++j) w.g[j] = make_float2(g[j], g[j]);
+  for (int j = 0; j <= c; ++j) w.g[KT - c + j] = make_float2(g[j], g[j]);
   return w;
 }
 
@@ -1256,24 +1262,34 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// The TMA-staged axial pass applies when the FP32 working sinogram can be
-// described as a 2D tensor of n^2 planes of J bins (16-byte aligned base,
-// plane pitch J * 4 a multiple of 16 bytes), segments fit the shared-memory
-// tile (n_rings <= kTmaMaxRings), the window radius is instantiated, x T <
-// 2^32 for every bin x of a plane (exact LOR by multiply-high), and the
-// environment does not switch it off (PSC_AXIAL_TMA=0).  The map describes
-// 256-bin by 1-plane boxes.
+// The TMA-staged axial pass applies when segments fit the shared-memory tile
+// (n_rings <= kTmaMaxRings), the radius is at most kWideRadius (448 x 45 without TOF,
+// radius 31: per-tap loop 19.2 ms, tiles 1.08 ms), x T < 2^32 for
+// every bin x of a plane (exact LOR by multiply-high), and the environment
+// does not switch it off (PSC_AXIAL_TMA=0); the working sinogram's planes then
+// have to start 16 bytes apart, so those of J bins with J not a multiple of 4 are
+// padded (odd view and TOF counts: 102 crystals x 45 rings, 27 TOF bins, radius 8:
+// direct pass 1068 us, tiles 717 us).  The map describes n^2 planes of J bins
+// in 256-bin by 1-plane boxes.
+long long finalize_pitch(const FinParams& p) {
+  const char* env = std::getenv("PSC_AXIAL_TMA");
+  const long long J = (long long)p.V * p.R * p.T;
+  const bool tiles = !(env && env[0] == '0') && p.K[2] <= kWideRadius && p.n_rings <= kTmaMaxRings &&
+                     J * p.T < (1LL << 32) && tensor_map_encoder();
+  return tiles ? (J + 3) / 4 * 4 : J;
+}
+
 static bool axial_tma_map(const FinParams& p, CUtensorMap* map, int tw) {
   const char* env = std::getenv("PSC_AXIAL_TMA");
   if (env && env[0] == '0') return false;
   const long long J = (long long)p.V * p.R * p.T;
-  if (p.KT[2] < 0 || p.n_rings > kTmaMaxRings || J % 4 != 0 || J * p.T >= (1LL << 32) ||
+  if (p.K[2] > kWideRadius || p.n_rings > kTmaMaxRings || p.pitch % 4 != 0 || J * p.T >= (1LL << 32) ||
       ((uintptr_t)p.scratch & 15) != 0)
     return false;
   const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
   if (!encode) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)J, (cuuint64_t)p.n_rings * (cuuint64_t)p.n_rings};
-  const cuuint64_t strides[1] = {(cuuint64_t)J * sizeof(float)};
+  const cuuint64_t strides[1] = {(cuuint64_t)p.pitch * sizeof(float)};
   const cuuint32_t box[2] = {(cuuint32_t)tw, 1};
   const cuuint32_t elem[2] = {1, 1};
   return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, p.scratch, dims, strides, box, elem,
@@ -1287,7 +1303,7 @@ static cudaError_t run_axial_tma(const FinParams& p, const CUtensorMap& map, dim
   auto k = smooth_axial_tma_kernel<KT, kDivide, kNorm, kFault, TW>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<grid, TW / 2, smem, s>>>(p, map, pair_weights<KT>(p.g[2]));
+  k<<<grid, TW / 2, smem, s>>>(p, map, pair_weights<KT>(p.g[2], p.KT[2] >= 0 ? KT : p.K[2]));
   return cudaGetLastError();
 }
 
@@ -1320,7 +1336,7 @@ cudaError_t launch_smooth_axial(const FinParams& p, int lo, int hi, cudaStream_t
       constexpr int kNarrow = kSmoothThreads / 2;
       const dim3 grid((unsigned)((J + (narrow ? kNarrow : kSmoothThreads) - 1) / (narrow ? kNarrow : kSmoothThreads)),
                       (unsigned)(b - a));
-      const cudaError_t e = for_window_radius(p.KT[2], [&](auto kt) -> cudaError_t {
+      auto run = [&](auto kt) -> cudaError_t {
         constexpr int KT = decltype(kt)::value;
         if constexpr (KT == 8)
           if (fault)
@@ -1334,11 +1350,14 @@ cudaError_t launch_smooth_axial(const FinParams& p, int lo, int hi, cudaStream_t
         if (p.divide_acc) return run_axial_tma<KT, true, false>(q, map, grid, rows, s);
         if (p.rnorm) return run_axial_tma<KT, false, true>(q, map, grid, rows, s);
         return run_axial_tma<KT, false, false>(q, map, grid, rows, s);
-      });
+      };
+      const cudaError_t e = p.KT[2] >= 0 ? for_window_radius(p.KT[2], run)
+                                         : run(std::integral_constant<int, kWideRadius>{});
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
   }
+  if (p.pitch != (long long)p.V * p.R * p.T) return cudaErrorInvalidValue;  // padded for tiles that could not be described
   return dispatch_kt<AxialL>(p.KT[2], q, dim3(smooth_blocks((long long)p.R * p.T), (unsigned)((hi - lo) * p.V)), s);
 }
 

@@ -114,6 +114,7 @@ extern "C" int psc_finalize_static(const int64_t* acc, int32_t n_rings, int32_t 
     base = g_scratch_ptr[dev];
   }
   p.scratch = (float*)base;
+  p.pitch = J;
   if (norm) {
     double* rnorm = (double*)((unsigned char*)base + norm_off);
     p.norm = norm;

@@ -19,7 +19,8 @@ int set_error(int code, const char* msg);
 struct FinParams {
   const long long* acc;
   double* out;
-  float* scratch;              // FP32 working sinogram, n_bins floats (smoothing only)
+  float* scratch;              // FP32 working sinogram, n_rings^2 planes `pitch` floats apart (smoothing only)
+  long long pitch;             // V R T, or more (finalize_pitch)
   const double* sens;
   const double* norm;
   const double* rnorm;         // 1/norm (FP64), 0 where norm == 0: the smoothed epilogue's factor
@@ -61,6 +62,8 @@ cudaError_t transport_occupancy(int lut_dtype, int block, size_t smem, int* bloc
 // smoothing weights and window radii from sigma (bins, per axis): PSC_OK,
 // or an error code with the message set
 int finalize_plan(FinParams& p, const double sigma[3]);
+// the plane pitch of the working sinogram that lets a planned call take its fastest axial pass
+long long finalize_pitch(const FinParams& p);
 cudaError_t launch_finalize(const FinParams& p, int sms, cudaStream_t s);
 // the parts of launch_finalize: the unsmoothed product over planes [lo, hi);
 // the radial and view passes over every plane; the axial pass (with the

@@ -1510,7 +1510,10 @@ static int finalize_launches(psc_ctx* ctx, const psc_finalize_args* a, double* o
     return fail(PSC_EINVAL, "in a stream capture the copies to host memory run on the capturing stream");
   {
     std::lock_guard<std::mutex> lk(ctx->scratch_mu);
+    // it grows when a sinogram's bins do not fit (never for a plane pitch alone: a
+    // captured call keeps its address), with room for padded planes
     const size_t need = sizeof(float) * (size_t)p.n_bins;
+    const size_t padded = sizeof(float) * (size_t)((long long)nr * nr * ((J + 3) / 4 * 4));
     if (ctx->scratch.bytes < need) {
       if (cap) return fail(PSC_EINVAL, "the smoothing scratch grows outside a capture: run the call once first");
       cudaStreamSynchronize(s);
@@ -1520,15 +1523,23 @@ static int finalize_launches(psc_ctx* ctx, const psc_finalize_args* a, double* o
         ctx->scratch.p = nullptr;
         ctx->scratch.bytes = 0;
       }
-      cudaError_t e = cudaMalloc(&ctx->scratch.p, need);
+      size_t got = padded;
+      cudaError_t e = cudaMalloc(&ctx->scratch.p, got);
+      if (e != cudaSuccess && padded > need) {
+        cudaGetLastError();
+        got = need;
+        e = cudaMalloc(&ctx->scratch.p, got);
+      }
       if (e != cudaSuccess) {
         cudaGetLastError();
         ctx->scratch.p = nullptr;
         return fail(PSC_ENOMEM, "finalize scratch of %zu bytes: %s", need, cudaGetErrorString(e));
       }
-      ctx->scratch.bytes = need;
+      ctx->scratch.bytes = got;
     }
     p.scratch = (float*)ctx->scratch.p;
+    p.pitch = finalize_pitch(p);
+    if (sizeof(float) * (size_t)((long long)nr * nr * p.pitch) > ctx->scratch.bytes) p.pitch = J;
     if (!cap) CK(cudaStreamWaitEvent(s, ctx->scratch_done, 0), "order scratch users");
     if (!hc) {
       CK(launch_finalize(p, ctx->sms, s), "finalize");

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n_rings", [1, 8, 9, 17, 37])        # segments of 1 .. 37 planes: whole and partial blocks, both tile widths
-@pytest.mark.parametrize("radius", [1, 7, 8, 10, 20, 24])     # also windows longer than the segment
+@pytest.mark.parametrize("radius", [1, 7, 8, 10, 20, 24, 25, 31, 32])     # also windows longer than the segment
 @pytest.mark.parametrize("offset", [0, 1])                    # an estimate on a 16-byte boundary, and 8 bytes past one
 def test_pairs_equal_direct_pass(n_rings, radius, offset, monkeypatch):
     import torch
@@ -37,6 +37,32 @@ def test_pairs_equal_direct_pass(n_rings, radius, offset, monkeypatch):
                 psc.psc_finalize(f.ctx, psc.finalize_args(f.a_id, **kw, **extra), out, stream)
                 torch.cuda.synchronize()
                 got.append(out.cpu().numpy().view(np.int64))
+            np.testing.assert_array_equal(got[0], got[1])
+    finally:
+        f.close()
+
+
+@pytest.mark.parametrize("n_crystals,n_rad,n_tof", [(10, 9, 5), (10, 9, 1), (12, 7, 3), (38, 33, 27)])  # planes of 225, 45, 126, 16929 bins
+@pytest.mark.parametrize("radius", [3, 31])
+@pytest.mark.parametrize("value", [1.0, np.inf])              # an infinite factor spreads over the window and no further
+def test_padded_planes_equal_direct_pass(n_crystals, n_rad, n_tof, radius, value, monkeypatch):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    sc = W.scanner_small(n_crystals=n_crystals, n_rings=37, n_tof=n_tof, n_rad=n_rad)
+    f = Fin(sc)
+    try:
+        rng = np.random.default_rng(radius)
+        acc = rng.integers(1, 1 << 40, size=sc.shape, dtype=np.int64)
+        f.write_acc(acc)
+        sens = rng.uniform(0.5, 1.5, size=sc.shape)
+        sens[18 * 37 + 18, 1, 2, 0] = value
+        sid = f.sino(sens, False)
+        for first in (True, False):
+            got = []
+            for tma in ("1", "0"):
+                monkeypatch.setenv("PSC_AXIAL_TMA", tma)
+                got.append(f.run(sens=sid, sens_first=first, sigma=(0.5, 0.5, radius / 4.0), scale=0.37).cpu().numpy())
             np.testing.assert_array_equal(got[0], got[1])
     finally:
         f.close()
