@@ -8,12 +8,14 @@
 // is exact to the last bit).
 //
 // With smoothing three separable passes, each reading and writing every bin
-// once.  A thread owns one column of the smoothed axis and slides down it
-// with a register window: NB outputs per step from NB new loads, the 2K
-// halo rows carried over in registers, the reflected edge rows loaded by
-// index.  Loads and stores of a warp cover 32 consecutive bins of the
-// innermost axes, so every access is coalesced; no shared memory and no
-// barriers are needed, and enough warps are resident to keep HBM busy.
+// once.  The axial pass, and the radial pass of short TOF axes and small
+// sinograms, work on shared-memory tiles (below).  Elsewhere a thread owns one
+// column of the smoothed axis and slides down it with a register window: NB
+// outputs per step from NB new loads, the 2K halo rows carried over in
+// registers, the reflected edge rows loaded by index.  Loads and stores of a
+// warp cover 32 consecutive bins of the innermost axes, so every access is
+// coalesced; no shared memory and no barriers are needed, and enough warps
+// are resident to keep HBM busy.
 //   A  radial: acc (int64) -> FP32, columns (plane, view, tof) along rad,
 //              into the first half of the output buffer (used as scratch)
 //   B  view:   that -> FP32 working sinogram, columns (plane, rad, tof)
@@ -23,8 +25,9 @@
 //              segment's planes
 // No pass writes what it reads.  Kernels are truncated at ceil(4 sigma) with
 // weights normalised to 1 and zero-padded to the instantiated radius KT
-// (exact for K <= 8, then 10, 12, 16, 20, 24; a per-tap loop beyond), so the
-// FMA chain is the same for every KT >= K; edges reflect half-sample
+// (exact for K <= 8, then 10, 12, 16, 20, 24; beyond, the axial tiles to radius
+// 32 and else a per-tap loop read no tap beyond K), so the FMA chain is the
+// same for every KT >= K; edges reflect half-sample
 // symmetrically; a plane's axial neighbours are the planes of the same ring
 // difference.
 #include <algorithm>
@@ -500,7 +503,8 @@ __global__ void __launch_bounds__(kSmoothThreads) smooth_radial_kernel(const __g
 }
 
 // ---------------------------------------------------------------------------
-// pass A for short TOF axes: whole radial lines staged in shared memory.
+// pass A for short TOF axes and small sinograms: whole radial lines staged in
+// shared memory.
 // A column's neighbours along rad lie T bins apart, so with few TOF bins the
 // kernel above touches a new sector per thread and load, and a plane has few
 // columns: without TOF it moved 2.4 GB in 1.77 ms.  Here a CTA takes G pairs of
@@ -514,10 +518,15 @@ __global__ void __launch_bounds__(kSmoothThreads) smooth_radial_kernel(const __g
 // the host so that a half-warp's lanes (block, tof) read different banks.
 // Radius 8, 448 x 45 scanner, radial pass: 1 TOF bin 1798 -> 572 us (with one
 // line a thread 896), 3 TOF bins 2088 -> 1737 us, 5 TOF bins 2523 -> 2889 us:
-// taken up to kLineMaxT TOF bins.
+// taken up to kLineMaxT TOF bins.  A sinogram with few columns (planes x views x TOF
+// bins) leaves the column kernel too few threads, each with a whole line to walk, so
+// below kFewColumns any TOF axis takes this one: 64 x 8 scanner, 7 bins (14 K columns) 13 ->
+// 6 us; 300 x 8, 5 bins (48 K) 69 -> 46; 100 x 20, 9 bins (180 K) 66 -> 58; 300 x
+// 16, 5 bins (192 K) 194 -> 167; 200 x 16, 9 bins (230 K) 130 against 136 us.
 // grid (ceil(V / (2 G)), planes)
 // ---------------------------------------------------------------------------
 constexpr int kLineMaxT = 4;
+constexpr long long kFewColumns = 200000;
 constexpr int kLineThreads = 512, kLineCtas = 2;
 struct LineStage {
   int G;            // pairs of lines per CTA
@@ -1202,13 +1211,15 @@ static cudaError_t for_window_radius(int kt, F&& f) {
   }
 }
 
-// The staged radial pass takes short TOF axes whose lines fit a CTA: an
+// The staged radial pass takes short TOF axes, and any where the columns are few,
+// whose lines fit a CTA: an
 // instantiated radius no larger than the line (one reflection), at most 512
 // threads of 8 x 2 outputs, 100 KB of shared memory, and exact divisions by
 // multiply-high.
 static bool line_stage(const FinParams& p, LineStage* h) {
   const int KT = p.KT[0], R = p.R, T = p.T;
-  if (KT < 0 || R < KT || T > kLineMaxT) return false;
+  if (KT < 0 || R < KT) return false;
+  if (T > kLineMaxT && (long long)finalize_planes(p) * p.V * T > kFewColumns) return false;
   const int RB = (R + 7) / 8, items = RB * T;
   if (items > kLineThreads) return false;
   h->RB = RB;
@@ -1336,7 +1347,7 @@ cudaError_t launch_smooth_axial(const FinParams& p, int lo, int hi, cudaStream_t
     // segments of at most kTmaShortRows planes in launches of their own,
     // whose smaller tiles let 6 CTAs share an SM's shared memory; the long
     // middle segments run tiles half as wide (128 bins, half the shared
-    // memory per CTA) in CTAs of 128 threads
+    // memory per CTA) in CTAs of 64 threads
     const int n = p.n_rings, S = std::min(kTmaShortRows, n);
     const int c1 = std::max(lo, std::min(hi, S)), c2 = std::max(c1, std::min(hi, 2 * n - 1 - S));
     const int cuts[4] = {lo, c1, c2, hi};

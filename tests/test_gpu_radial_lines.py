@@ -13,8 +13,10 @@ pytestmark = pytest.mark.gpu
 
 
 # crystals, radial bins, TOF bins: odd and even view counts (a pair without its second line), lines of one partial
-# block of 8 rows, several CTAs a plane, the longest TOF axis taken and the shortest that is not
-@pytest.mark.parametrize("n_crystals,n_rad,n_tof", [(8, 7, 1), (10, 9, 3), (46, 33, 1), (46, 45, 4), (200, 199, 1), (44, 41, 5)])
+# block of 8 rows, several CTAs a plane, longer TOF axes of small sinograms, and one of 224,000 columns, which the
+# column kernel takes as a whole and this one for the segment range
+@pytest.mark.parametrize("n_crystals,n_rad,n_tof", [(8, 7, 1), (10, 9, 3), (46, 33, 1), (46, 45, 4), (200, 199, 1), (44, 41, 5),
+                                                     (22, 21, 27), (200, 9, 140)])
 @pytest.mark.parametrize("radius", [0, 1, 5, 7])     # at most the shortest line
 @pytest.mark.parametrize("factors", [None, "sens_first", "norm"])
 def test_lines_match_oracle(n_crystals, n_rad, n_tof, radius, factors):
