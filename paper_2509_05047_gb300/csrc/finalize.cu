@@ -315,13 +315,17 @@ __device__ __noinline__ double plain_bin_general(unsigned long long u, double c,
 // three times as long as the memory, so the significands are multiplied on the
 // integer pipes without leaving their unpacked form (about 65 instructions a
 // bin; bins without an event, most of them, skip the products).  A thread has
-// four bins in flight, 256 apart: with one at a time and packed intermediates
+// eight bins in flight, 256 apart: with one at a time and packed intermediates
 // (integer products of 64-bit halves, rounding by variable shifts) the kernel
-// waited on memory and on itself.  288 x 16 scanner, 13 TOF bins, per-LOR
-// sensitivity (137.5 M bins, 2.29 GB): 1330 -> 490 us with 2 % of the bins
-// filled, 1506 -> 756 us with all of them.
+// waited on memory and on itself.  Each lane then takes its own next filled bin,
+// whichever of the eight it is: a pass over the products for every bin that any
+// lane of the warp has filled ran them nearly half-empty twice per four bins.
+// Where all lanes have more than four filled, the eight are taken in order.
+// 288 x 16 scanner, 13 TOF bins, per-LOR sensitivity (137.5 M bins, 2.29 GB): 1330 us
+// at first, 490 us with four bins in order, 387 us now with 2 % of the bins
+// filled; 1506, 756 and 792 us with all of them.
 // ---------------------------------------------------------------------------
-constexpr int kPlainBins = 4;
+constexpr int kPlainBins = 8;
 
 __global__ void __launch_bounds__(256) finalize_plain_kernel(const __grid_constant__ FinParams P) {
   // grid.y = plane, grid.x strides over the plane's J = V * R * T bins
@@ -351,29 +355,48 @@ __global__ void __launch_bounds__(256) finalize_plain_kernel(const __grid_consta
                                               : (long long)j));
       }
     }
+    // bins without counts are zeros; the others of a lane wait in `filled`
+    unsigned filled = 0;
 #pragma unroll
     for (int q = 0; q < kPlainBins; ++q) {
       const int j = j0 + 256 * q;
-      if (j >= J) break;
       const unsigned s_hi = (unsigned)((unsigned long long)__double_as_longlong(s[q]) >> 32);
-      const unsigned sign = c_sign ^ (s_hi & 0x80000000u);
-      const unsigned s_exp = (s_hi >> 20) & 0x7ffu;
-      double x;
-      if (u[q] == 0 && s_exp != 0x7ffu) {
-        x = __hiloint2double((int)sign, 0);
-      } else if ((u[q] >> 53) != 0 || u[q] == 0 || !c_normal || s_exp - 1u >= 0x7feu) {
-        x = plain_bin_general(u[q], P.c, s[q], sens != nullptr);
-      } else {
-        const int lz = __clzll((long long)u[q]);
-        const unsigned long long m = u[q] << (lz - 11);
-        Sig r = sig_mul(Sig{(unsigned)(m >> 32), (unsigned)m, 63 - lz}, c);
-        bool normal = r.e > -1023 && r.e < 1024;
-        if (sens) r = sig_mul(r, sig_of(s[q]));
-        normal = normal && r.e > -1023 && r.e < 1024;
-        x = __hiloint2double((int)(sign | (((unsigned)(r.e + 1022) << 20) + r.hi)), (int)r.lo);
-        if (!normal) x = plain_bin_general(u[q], P.c, s[q], sens != nullptr);
+      if (u[q] != 0 || ((s_hi >> 20) & 0x7ffu) == 0x7ffu) {
+        filled |= j < J ? 1u << q : 0u;
+      } else if (j < J) {
+        out[j] = __hiloint2double((int)((c_sign ^ s_hi) & 0x80000000u), 0);
       }
-      out[j] = x;
+    }
+    auto product = [&](unsigned long long v, double f) -> double {
+      const unsigned s_hi = (unsigned)((unsigned long long)__double_as_longlong(f) >> 32);
+      if ((v >> 53) != 0 || v == 0 || !c_normal || ((s_hi >> 20) & 0x7ffu) - 1u >= 0x7feu)
+        return plain_bin_general(v, P.c, f, sens != nullptr);
+      const int lz = __clzll((long long)v);
+      const unsigned long long m = v << (lz - 11);
+      Sig r = sig_mul(Sig{(unsigned)(m >> 32), (unsigned)m, 63 - lz}, c);
+      bool normal = r.e > -1023 && r.e < 1024;
+      if (sens) r = sig_mul(r, sig_of(f));
+      normal = normal && r.e > -1023 && r.e < 1024;
+      if (!normal) return plain_bin_general(v, P.c, f, sens != nullptr);
+      return __hiloint2double((int)(((c_sign ^ s_hi) & 0x80000000u) | (((unsigned)(r.e + 1022) << 20) + r.hi)), (int)r.lo);
+    };
+    if (__all_sync(__activemask(), __popc(filled) > kPlainBins / 2)) {
+#pragma unroll
+      for (int q = 0; q < kPlainBins; ++q)
+        if (filled >> q & 1u) out[j0 + 256 * q] = product(u[q], s[q]);
+      continue;
+    }
+    while (filled) {  // each lane's next filled bin: the lanes' bins need not be the same ones
+      const int q = __ffs((int)filled) - 1;
+      filled &= filled - 1u;
+      unsigned long long v = u[0];
+      double f = s[0];
+#pragma unroll
+      for (int i = 1; i < kPlainBins; ++i) {
+        v = q == i ? u[i] : v;
+        f = q == i ? s[i] : f;
+      }
+      out[j0 + 256 * q] = product(v, f);
     }
   }
 }

@@ -44,3 +44,26 @@ def test_products_are_ieee(n_tof, per_lor, scale):
         np.testing.assert_array_equal(got.view(np.int64)[~nan], exp.view(np.int64)[~nan])
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("density", [1.0, 0.6, 0.05, 0.0])   # all of a lane's bins filled, about half, few, none
+@pytest.mark.parametrize("n_tof", [1, 5])                    # 627 and 3135 bins a plane: less and more than a CTA's 2048
+def test_filled_bins_in_any_number(density, n_tof):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    sc = W.scanner_small(n_crystals=38, n_rings=3, n_tof=n_tof, n_rad=33)
+    f = Fin(sc)
+    try:
+        rng = np.random.default_rng(8)
+        acc = rng.integers(1, 1 << 40, size=sc.shape)
+        acc[rng.uniform(size=sc.shape) >= density] = 0
+        sens = rng.uniform(0.5, 1.5, size=sc.lor_shape)
+        sens.ravel()[::97] = np.inf
+        f.write_acc(acc)
+        with np.errstate(all="ignore"):
+            exp = (acc.astype(np.float64) * math.ldexp(0.37, -32)) * sens[..., None]
+        got = f.run(sens=f.sino(sens, True), scale=0.37).cpu().numpy()
+        np.testing.assert_array_equal(got, exp)
+    finally:
+        f.close()
