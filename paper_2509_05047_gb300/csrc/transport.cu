@@ -414,6 +414,16 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
       const int g = lane_id < (kmax >> 3) ? (int)dbg_idx(B.dbg, kSiteSlot, s_sel[warp][lane_id], n_slots) : -1;
       __syncwarp();
 
+      // In EMIT a slot takes the work item's next history, if there is one.  Loop control
+      // has to be the same in all lanes, so the end of the item is voted on, from the
+      // values that the lanes' own atomics returned: another warp may move s_next between
+      // two lanes' reads of it.
+      unsigned off = ~0u;
+      if (sec == kEmit) {
+        if (g >= 0) off = atomicAdd(&s_next, 1u);
+        if (__any_sync(0xffffffffu, off + 1u >= s_len)) waiting = ~0xffu;
+      }
+
       if (g >= 0) {
         uint32_t m = s_meta[g];
         auto history = [&]() -> unsigned long long { return s_lo + (m >> kMetaHistory); };
@@ -458,8 +468,6 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
         };
 
         // ---- emission (stream 0, words 0..6) ----
-        // (the slot takes the work item's next history, if there is one)
-        const unsigned off = sec == kEmit ? atomicAdd(&s_next, 1u) : ~0u;
         const bool emitted = off < s_len;
         float4 pos, dir;
         if (emitted) {
@@ -820,7 +828,6 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
         }
       }
       __syncwarp();  // slot updates are visible to the lanes that vote on them next
-      if (sec == kEmit && s_next >= s_len) waiting = ~0xffu;
     }
 
     __syncthreads();  // every slot is done with the chunk before the next fetch
