@@ -551,6 +551,7 @@ __global__ void __launch_bounds__(kSmoothThreads) smooth_radial_kernel(const __g
 constexpr int kLineMaxT = 4;
 constexpr long long kFewColumns = 200000;
 constexpr int kLineThreads = 512, kLineCtas = 2;
+constexpr int kLineSmem = 100 * 1024;  // a CTA's lines at most
 struct LineStage {
   int G;            // pairs of lines per CTA
   int RB;           // output blocks of 8 rows a line
@@ -1261,7 +1262,7 @@ static bool line_stage(const FinParams& p, LineStage* h) {
   }
   h->LP = (R + 2 * KT + 7 + 7) / 8 * h->S;  // the last block's rows reach 8 RB - 1 + 2 KT <= R + 6 + 2 KT
   const long long n = (long long)h->G * R * T + kLineThreads * 8;
-  if ((size_t)h->G * h->LP * sizeof(float2) > 100 * 1024) return false;
+  if ((size_t)h->G * h->LP * sizeof(float2) > (size_t)kLineSmem) return false;
   if (n * R * T >= (1LL << 32) || ((long long)R + 2 * KT) * T * 8 * T >= (1LL << 32) || (kLineThreads + 31LL) * items >= (1LL << 32))
     return false;
   auto magic = [](int d) { return d == 1 ? 0u : (unsigned)(((1ULL << 32) + d - 1) / d); };
@@ -1284,7 +1285,9 @@ cudaError_t launch_smooth_front(const FinParams& p, cudaStream_t s) {
       constexpr int KT = decltype(kt)::value;
       const auto k = (p.sens_first && p.sens) || p.norm ? smooth_radial_lines_kernel<KT, true>
                                                         : smooth_radial_lines_kernel<KT, false>;
-      const cudaError_t a = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      // the limit belongs to the kernel on its device, not to this launch: always the same
+      // one, so that no thread lowers it between another's call and launch
+      const cudaError_t a = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem);
       if (a != cudaSuccess) return a;
       k<<<grid, threads, smem, s>>>(p, h, pair_weights<KT>(p.g[0]));
       return cudaGetLastError();
@@ -1350,7 +1353,9 @@ template <int KT, bool kDivide, bool kNorm, bool kFault = false, int TW = kSmoot
 static cudaError_t run_axial_tma(const FinParams& p, const CUtensorMap& map, dim3 grid, int rows, cudaStream_t s) {
   const size_t smem = (size_t)rows * TW * sizeof(float);
   auto k = smooth_axial_tma_kernel<KT, kDivide, kNorm, kFault, TW>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the largest tile of this width, whatever the launch's: the limit is shared with other threads' launches
+  constexpr int kMost = (TW == kSmoothThreads ? kTmaShortRows : kTmaMaxRings) * TW * (int)sizeof(float);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
   if (e != cudaSuccess) return e;
   k<<<grid, TW / 2, smem, s>>>(p, map, pair_weights<KT>(p.g[2], p.KT[2] >= 0 ? KT : p.K[2]));
   return cudaGetLastError();

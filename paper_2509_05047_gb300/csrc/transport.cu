@@ -848,10 +848,23 @@ size_t transport_smem_bytes(const PhantomParams& ph, int block) {
          sizeof(float4) * (size_t)ph.n_mat * ph.n_tab + sizeof(float) * (ph.n_tab + kMaxMaterials);
 }
 
+// Lets a kernel use all the dynamic shared memory that the device has for it.  The limit
+// belongs to the kernel on its device: set to each launch's own size, one thread could
+// lower it between another's call and launch.
+template <class K>
+static cudaError_t allow_smem(K kernel) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+}
+
 template <int DT, bool kDebug, bool kOneJob = false, bool kFixed = false>
 static cudaError_t launch_dt(const BatchParams& p, int grid, int block, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(transport_kernel<DT, kDebug, kOneJob, kFixed>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(transport_kernel<DT, kDebug, kOneJob, kFixed>);
   if (e != cudaSuccess) return e;
   transport_kernel<DT, kDebug, kOneJob, kFixed><<<grid, block, smem, s>>>(p);
   return cudaGetLastError();
@@ -886,8 +899,7 @@ cudaError_t launch_transport(const BatchParams& p, int lut_dtype, int grid, int 
 // kernel would size its grid for one CTA per SM).
 template <int DT>
 static cudaError_t occupancy_dt(int block, size_t smem, int* blocks_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(transport_kernel<DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  const cudaError_t e = allow_smem(transport_kernel<DT, false>);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, transport_kernel<DT, false>, block, smem);
 }
