@@ -58,7 +58,6 @@ __device__ __forceinline__ long long dbg_idx(DebugRecord* rec, unsigned site, lo
 
 constexpr int kMaxMaterials = 8;
 constexpr int kMaxSteps = 4096;     // Woodcock steps per photon (safety bound)
-constexpr unsigned long long kMaxChunk = 1ull << 16;  // histories of a work item (a slot holds 16 bits of the index)
 constexpr int kMaxTries = 64;       // rejection-sampling tries, last proposal kept
 constexpr float kPolarEps = 1e-6f;  // |d_z| > 1 - eps: rotate about the z axis
 constexpr float kRestKeV = 511.0f;

@@ -29,6 +29,7 @@
 
 #include "psc.h"
 #include "psc_internal.h"
+#include "work_items.h"
 
 using namespace psc;
 
@@ -1134,27 +1135,9 @@ static int batch_impl(psc_ctx* ctx, const psc_sim_args* args, int32_t n, psc_sta
       CK(transport_occupancy(dt, block, smem, &per_sm), "occupancy");
       grid = ctx->sms * std::max(per_sm, 1);
     }
-    // Work items.  A CTA that ends an item drains its slots before it takes the
-    // next one (about 30 us beside its neighbours), and items left over after
-    // whole rounds of the grid run on an idle chip.  So each request is cut into
-    // the fewest equal items that fill whole rounds (chunks_per_cta of them at
-    // least, at most max_chunk histories each), the largest request first, so
-    // that the small items come last.  Against two or more items a CTA of at
-    // least 1024 histories: small scanner, 1e6 histories 121 -> 88 us, 2e4 39 ->
-    // 32 us; 1e8 through the gaps scanner (5.02 rounds of 65536 before, now 6 of
-    // 54826) 7.82 -> 7.13 ms; six uneven requests 7.35 -> 7.25 ms.  Items of a
-    // batch are not cut below 1/32 of a CTA's share of all its histories: 32
-    // uneven requests 7.66 ms, at 1/128 7.79 ms.
-    constexpr unsigned long long kMinChunk = 128, kBatchItems = 32;
-    const unsigned long long g_ = (unsigned long long)grid;
-    const unsigned long long most = std::min(kMaxChunk, std::max<unsigned long long>(1024, sc_in.max_chunk));
-    unsigned long long all = 0;
+    // the largest request first, so that the small items come last
     std::vector<int> order(bp.n_jobs);
-    for (int j = 0; j < bp.n_jobs; ++j) {
-      order[j] = j;
-      all += bp.jobs[j].n / (g_ * kBatchItems);  // (per item: the sum of all histories may exceed 64 bits)
-    }
-    const unsigned long long least = std::max(kMinChunk, bp.n_jobs > 1 ? all : 0);
+    for (int j = 0; j < bp.n_jobs; ++j) order[j] = j;
     if (bp.n_jobs > 1) {
       const std::vector<Job> jb(bp.jobs, bp.jobs + bp.n_jobs);
       const std::vector<ListmodeOut> lm(bp.lm, bp.lm + bp.n_jobs);
@@ -1164,13 +1147,13 @@ static int batch_impl(psc_ctx* ctx, const psc_sim_args* args, int32_t n, psc_sta
         bp.lm[j] = lm[order[j]];
       }
     }
+    unsigned long long histories[kMaxJobs], chunk[kMaxJobs];
+    for (int j = 0; j < bp.n_jobs; ++j) histories[j] = bp.jobs[j].n;
+    work_items(histories, bp.n_jobs, (unsigned long long)grid, (unsigned long long)sc_in.chunks_per_cta, sc_in.max_chunk,
+               chunk);
     for (int j = 0; j < bp.n_jobs; ++j) {
       Job& jb = bp.jobs[j];
-      const unsigned long long per_cta = jb.n / g_ + (jb.n % g_ != 0);
-      const unsigned long long rounds = std::max<unsigned long long>(sc_in.chunks_per_cta, per_cta / most + (per_cta % most != 0));
-      const unsigned long long per = std::min(most, std::max(least, per_cta / rounds + (per_cta % rounds != 0)));
-      const unsigned long long items = jb.n / per + (jb.n % per != 0);
-      jb.chunk = jb.n / items + (jb.n % items != 0);
+      jb.chunk = chunk[j];
       total += jb.n / jb.chunk + (jb.n % jb.chunk != 0);
       bp.chunk_end[j] = total;
     }
