@@ -985,8 +985,18 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
   for (int o0 = 0; o0 < L; o0 += NB) {
     const int rows = min(NB, L - o0);
     if (!need(min(o0 + NB - 1 + KT, L - 1))) return give_up();
-    // the block's factors, on their way during the FMA chains
+    // the block's factors (divisors), on their way during the FMA chains
     double fs[NB][2];
+    long long qa[NB][2];
+    if (kDivide) {
+#pragma unroll
+      for (int q = 0; q < NB; ++q)
+        if (q < rows) {
+          qa[q][0] = __ldg(ap + q * bin_step);
+          qa[q][1] = __ldg(ap + q * bin_step + two);
+        }
+      ap += NB * bin_step;
+    }
     if (!kDivide && use_sens) {
 #pragma unroll
       for (int q = 0; q < NB; ++q)
@@ -1020,18 +1030,13 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       if (q >= rows) break;
-      long long qa0 = 0, qa1 = 0;
       double fr0 = 1.0, fr1 = 1.0;
-      if (kDivide) {
-        qa0 = __ldg(ap + q * bin_step);
-        qa1 = __ldg(ap + q * bin_step + two);
-      }
       if (kNorm) {
         fr0 = __ldg(rp + q * rs);
         fr1 = __ldg(rp + q * rs + r1);
       }
-      const double e0 = axial_epilogue_fp64<kDivide, kNorm>(y[q].x, qa0, fr0, fs[q][0], use_sens, cf);
-      const double e1 = axial_epilogue_fp64<kDivide, kNorm>(y[q].y, qa1, fr1, fs[q][1], use_sens, cf);
+      const double e0 = axial_epilogue_fp64<kDivide, kNorm>(y[q].x, qa[q][0], fr0, fs[q][0], use_sens, cf);
+      const double e1 = axial_epilogue_fp64<kDivide, kNorm>(y[q].y, qa[q][1], fr1, fs[q][1], use_sens, cf);
       double* o = dst + q * bin_step;
       if (wide) {
         *reinterpret_cast<double2*>(o) = make_double2(e0, e1);
@@ -1041,7 +1046,6 @@ __global__ void __launch_bounds__(TW / 2, kTileThreads * 2 / TW)
       }
     }
     dst += NB * bin_step;
-    if (kDivide) ap += NB * bin_step;
     if (kNorm) rp += NB * rs;
   }
 }
