@@ -40,6 +40,7 @@
 #include <cudaTypedefs.h>
 
 #include "psc.h"
+#include "finalize_routes.h"
 #include "psc_internal.h"
 
 namespace psc {
@@ -1324,14 +1325,17 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 // every bin x of a plane (exact LOR by multiply-high), and the environment
 // does not switch it off (PSC_AXIAL_TMA=0); the working sinogram's planes then
 // have to start 16 bytes apart, so those of J bins with J not a multiple of 4 are
-// padded (odd view and TOF counts: 102 crystals x 45 rings, 27 TOF bins, radius 8:
-// direct pass 1068 us, tiles 717 us).  The map describes n^2 planes of J bins
-// in 256-bin by 1-plane boxes.
+// padded where that pays (odd view and TOF counts: 102 crystals x 45 rings, 27 TOF
+// bins, radius 8: direct pass 1068 us, tiles 717 us; where not: finalize_routes.h).
+// The map describes n^2 planes of J bins in 256-bin by 1-plane boxes.
 long long finalize_pitch(const FinParams& p) {
   const char* env = std::getenv("PSC_AXIAL_TMA");
   const long long J = (long long)p.V * p.R * p.T;
+  const long long segments = p.seg_hi <= p.seg_lo ? 2 * p.n_rings - 1 : p.seg_hi - p.seg_lo;
+  const AxialForm form = p.divide_acc ? kAxialDivide : p.rnorm ? kAxialNorm : kAxialPlain;
   const bool tiles = !(env && env[0] == '0') && p.K[2] <= kWideRadius && p.n_rings <= kTmaMaxRings &&
-                     J * p.T < (1LL << 32) && tensor_map_encoder();
+                     J * p.T < (1LL << 32) && padded_tiles_pay(p.K[2], form, p.n_rings, segments * J) &&
+                     tensor_map_encoder();
   return tiles ? (J + 3) / 4 * 4 : J;
 }
 

@@ -1,0 +1,36 @@
+// finalize_routes.h -- which of two kernels with the same results a smoothing
+// pass takes, where the line between them is a measurement (host code, no CUDA:
+// also compiled by the CPU tests).
+#ifndef PSC_FINALIZE_ROUTES_H
+#define PSC_FINALIZE_ROUTES_H
+
+namespace psc {
+
+// The axial pass of planes whose bins are not a multiple of 4: tiles on padded
+// planes, or the pass that loads its rows directly.  A tile reads its rows once,
+// and each output's 2 K + 1 taps from shared memory, where the direct pass moves a
+// register window; but a CTA sets up barriers, a row table and its copies first,
+// and a tile has one thread for two columns.  So tiles pay for wide windows and
+// where there are many columns (segments x bins of a plane) to hide the set-up.
+// Time of the whole call with tiles over that with the direct pass (8 to 90 rings, planes of
+// 45 to 140,000 bins):
+//   radius 25 - 32: 0.16 - 0.9 everywhere (direct: a load per tap)
+//   radius 16: 0.7 on average above 275,000 columns, 1.3 (up to 1.8) below
+//   radius 9 - 12: 0.8 above 700,000, 1.3 below; with a normalisation or its division (one
+//     more load an output, fewer tiles of more than 48 rows at once) 1.05 - 1.2 at 64 and 90 rings
+//   radius 3 - 8: 0.9 above 700,000 and up to 64 rings (48 with a normalisation), 1.1 - 1.4 below
+//     or at 90 rings; the division 1.1 - 1.6 everywhere
+//   radius 0 - 2: 1.0 at best; with a normalisation 0.9 above 700,000 and up to 48 rings
+enum AxialForm { kAxialPlain, kAxialNorm, kAxialDivide };
+
+inline bool padded_tiles_pay(int radius, AxialForm form, int n_rings, long long columns) {
+  if (radius > 24) return true;
+  if (radius > 12) return columns >= 275000;
+  if (form == kAxialDivide && radius <= 8) return false;
+  if (form == kAxialPlain && radius <= 2) return false;
+  return columns >= 700000 && n_rings <= (form != kAxialPlain ? 48 : radius > 8 ? 96 : 64);
+}
+
+}  // namespace psc
+
+#endif
