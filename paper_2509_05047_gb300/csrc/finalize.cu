@@ -1328,20 +1328,11 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 // padded where that pays (odd view and TOF counts: 102 crystals x 45 rings, 27 TOF
 // bins, radius 8: direct pass 1068 us, tiles 717 us; where not: finalize_routes.h).
 // The map describes n^2 planes of J bins in 256-bin by 1-plane boxes.
-long long finalize_pitch(const FinParams& p) {
-  const char* env = std::getenv("PSC_AXIAL_TMA");
-  const long long J = (long long)p.V * p.R * p.T;
-  const long long segments = p.seg_hi <= p.seg_lo ? 2 * p.n_rings - 1 : p.seg_hi - p.seg_lo;
-  const AxialForm form = p.divide_acc ? kAxialDivide : p.rnorm ? kAxialNorm : kAxialPlain;
-  const bool tiles = !(env && env[0] == '0') && p.K[2] <= kWideRadius && p.n_rings <= kTmaMaxRings &&
-                     J * p.T < (1LL << 32) && padded_tiles_pay(p.K[2], form, p.n_rings, segments * J) &&
-                     tensor_map_encoder();
-  return tiles ? (J + 3) / 4 * 4 : J;
-}
-
 static bool axial_tma_map(const FinParams& p, CUtensorMap* map, int tw) {
   const char* env = std::getenv("PSC_AXIAL_TMA");
   if (env && env[0] == '0') return false;
+  const char* inj = std::getenv("PSC_FAULT_TMA_MAP");  // tests: as if the planes could not be described
+  if (inj && inj[0] == '1') return false;
   const long long J = (long long)p.V * p.R * p.T;
   if (p.K[2] > kWideRadius || p.n_rings > kTmaMaxRings || p.pitch % 4 != 0 || J * p.T >= (1LL << 32) ||
       ((uintptr_t)p.scratch & 15) != 0)
@@ -1355,6 +1346,18 @@ static bool axial_tma_map(const FinParams& p, CUtensorMap* map, int tw) {
   return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, p.scratch, dims, strides, box, elem,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+long long finalize_pitch(const FinParams& p) {
+  const long long J = (long long)p.V * p.R * p.T;
+  const long long segments = p.seg_hi <= p.seg_lo ? 2 * p.n_rings - 1 : p.seg_hi - p.seg_lo;
+  const AxialForm form = p.divide_acc ? kAxialDivide : p.rnorm ? kAxialNorm : kAxialPlain;
+  if (J % 4 == 0 || !padded_tiles_pay(p.K[2], form, p.n_rings, segments * J)) return J;
+  // the other passes write padded planes only where the tiles can read them
+  FinParams q = p;
+  q.pitch = (J + 3) / 4 * 4;
+  CUtensorMap map;
+  return axial_tma_map(q, &map, kSmoothThreads) && axial_tma_map(q, &map, kSmoothThreads / 2) ? q.pitch : J;
 }
 
 template <int KT, bool kDivide, bool kNorm, bool kFault = false, int TW = kSmoothThreads>

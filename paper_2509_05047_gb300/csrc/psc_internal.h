@@ -62,7 +62,7 @@ cudaError_t transport_occupancy(int lut_dtype, int block, size_t smem, int* bloc
 // smoothing weights and window radii from sigma (bins, per axis): PSC_OK,
 // or an error code with the message set
 int finalize_plan(FinParams& p, const double sigma[3]);
-// the plane pitch of the working sinogram that lets a planned call take its fastest axial pass
+// the plane pitch of the working sinogram (p.scratch) that lets a planned call take its fastest axial pass
 long long finalize_pitch(const FinParams& p);
 cudaError_t launch_finalize(const FinParams& p, int sms, cudaStream_t s);
 // the parts of launch_finalize: the unsmoothed product over planes [lo, hi);

@@ -58,3 +58,26 @@ def test_tiles_equal_direct_pass(n_crystals, n_rad, n_tof, n_rings, radius, form
         assert torch.equal(got[0], got[1])
     finally:
         f.close()
+
+
+def test_planes_that_cannot_be_described_take_the_direct_pass(monkeypatch):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    for n_rad in (33, 32 + 5):    # odd planes that would be padded; the radius-31 window has no other instantiation
+        sc = W.scanner_small(n_crystals=38, n_rings=12, n_tof=5, n_rad=n_rad)
+        f = Fin(sc)
+        try:
+            acc = np.random.default_rng(n_rad).integers(0, 1 << 40, size=sc.shape, dtype=np.int64)
+            f.write_acc(acc)
+            got = []
+            for refused, kernel in (("0", "smooth_axial_tma_kernel"), ("1", "smooth_axial_kernel")):
+                monkeypatch.setenv("PSC_FAULT_TMA_MAP", refused)
+                out = torch.full(sc.shape, np.nan, dtype=torch.float64, device="cuda")
+                args = psc.finalize_args(f.a_id, sigma=(0.25, 0.25, 31 / 4.0), scale=0.37)
+                assert kernel in kernels_of(lambda stream: psc.psc_finalize(f.ctx, args, out, stream))
+                torch.cuda.synchronize()
+                got.append(out.view(torch.int64))
+            assert torch.equal(got[0], got[1])
+        finally:
+            f.close()
