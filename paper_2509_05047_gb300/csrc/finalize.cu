@@ -541,16 +541,12 @@ __global__ void __launch_bounds__(kSmoothThreads) smooth_radial_kernel(const __g
 // Rows lie in blocks of 8 rows of T values, block pitch S = 8 T + pad, chosen by
 // the host so that a half-warp's lanes (block, tof) read different banks.
 // Radius 8, 448 x 45 scanner, radial pass: 1 TOF bin 1798 -> 572 us (with one
-// line a thread 896), 3 TOF bins 2088 -> 1737 us, 5 TOF bins 2523 -> 2889 us:
-// taken up to kLineMaxT TOF bins.  A sinogram with few columns (planes x views x TOF
-// bins) leaves the column kernel too few threads, each with a whole line to walk, so
-// below kFewColumns any TOF axis takes this one: 64 x 8 scanner, 7 bins (14 K columns) 13 ->
-// 6 us; 300 x 8, 5 bins (48 K) 69 -> 46; 100 x 20, 9 bins (180 K) 66 -> 58; 300 x
-// 16, 5 bins (192 K) 194 -> 167; 200 x 16, 9 bins (230 K) 130 against 136 us.
+// line a thread 896), 3 TOF bins 2088 -> 1737 us, 5 TOF bins 2523 -> 2889 us; a sinogram
+// with few columns (planes x views x TOF bins) leaves the column kernel too few
+// threads, each with a whole line to walk: 64 x 8 scanner, 7 bins (14 K columns) 13 ->
+// 6 us; 300 x 8, 5 bins (48 K) 69 -> 46.  Which one a call takes: finalize_routes.h.
 // grid (ceil(V / (2 G)), planes)
 // ---------------------------------------------------------------------------
-constexpr int kLineMaxT = 4;
-constexpr long long kFewColumns = 200000;
 constexpr int kLineThreads = 512, kLineCtas = 2;
 constexpr int kLineSmem = 100 * 1024;  // a CTA's lines at most
 struct LineStage {
@@ -1240,15 +1236,14 @@ static cudaError_t for_window_radius(int kt, F&& f) {
   }
 }
 
-// The staged radial pass takes short TOF axes, and any where the columns are few,
-// whose lines fit a CTA: an
-// instantiated radius no larger than the line (one reflection), at most 512
+// The staged radial pass takes the calls it is the faster one for, whose lines fit a
+// CTA: an instantiated radius no larger than the line (one reflection), at most 512
 // threads of 8 x 2 outputs, 100 KB of shared memory, and exact divisions by
 // multiply-high.
 static bool line_stage(const FinParams& p, LineStage* h) {
   const int KT = p.KT[0], R = p.R, T = p.T;
   if (KT < 0 || R < KT) return false;
-  if (T > kLineMaxT && (long long)finalize_planes(p) * p.V * T > kFewColumns) return false;
+  if (!radial_lines_pay(T, (long long)finalize_planes(p) * p.V * T, p.K[0], (p.sens_first && p.sens) || p.norm)) return false;
   const int RB = (R + 7) / 8, items = RB * T;
   if (items > kLineThreads) return false;
   h->RB = RB;

@@ -31,6 +31,25 @@ inline bool padded_tiles_pay(int radius, AxialForm form, int n_rings, long long 
   return columns >= 700000 && n_rings <= (form != kAxialPlain ? 48 : radius > 8 ? 96 : 64);
 }
 
+// The radial pass: whole lines staged in shared memory, or a column a thread.
+// A column's neighbours lie T bins apart, so with few TOF bins a column's loads waste
+// sectors: up to 4 bins lines always pay (448 x 45, radius 8: 1 bin 1798 -> 572 us, 3 bins
+// 2088 -> 1737, 4 bins 0.97 - 0.99 of the whole call).  Above that the column pass is the better one
+// once its columns (planes x views x TOF bins) fill the chip; until then it walks whole lines
+// with too few threads.  Time of the whole call with lines over that with columns, 40 to 448
+// crystals, 5 to 60 TOF bins:
+//   below 75,000 columns: 0.7 - 1.0 (up to 1.11 at 27 bins without smoothing along rad)
+//   up to 200,000: radius 16 and up 0.6 - 0.9, 9 - 12 without a factor 0.7 - 1.0 to 120,000 and
+//     to 1.07 above; below radius 9 0.85 - 1.2 without a factor (worst between 85,000 and
+//     150,000); with a sensitivity or normalisation in the pass, which lines load
+//     together with the counts, 0.5 - 0.98 up to 20 bins, to 1.08 at 27
+inline bool radial_lines_pay(int T, long long columns, int radius, bool factors) {
+  if (T <= 4) return true;
+  if (radius > 12) return columns <= 200000;
+  if (T > 20 || (!factors && radius < 9)) return columns <= 75000;
+  return columns <= (factors ? 200000 : 120000);
+}
+
 }  // namespace psc
 
 #endif
