@@ -614,8 +614,10 @@ __global__ void __launch_bounds__(kLineThreads, kLineCtas)
           const float* a32 = with_sens ? P.sens32 : P.norm32;
           const double* a64 = with_sens ? P.sens : P.norm;
           const bool per_lor = with_sens ? P.sens_per_lor : P.norm_per_lor;
-          const long long at = per_lor ? dbg_idx(P.dbg, kSiteFinLor, lor, P.n_bins / T) : bin;
-          const long long at2 = per_lor ? dbg_idx(P.dbg, kSiteFinLor, lor + two * R, P.n_bins / T) : bin + two * RT;
+          const long long at = per_lor ? dbg_idx(P.dbg, kSiteFinLor, lor, P.n_bins / T)
+                                       : dbg_idx(P.dbg, kSiteFinBin, bin, P.n_bins);
+          const long long at2 = per_lor ? dbg_idx(P.dbg, kSiteFinLor, lor + two * R, P.n_bins / T)
+                                        : dbg_idx(P.dbg, kSiteFinBin, bin + two * RT, P.n_bins);
           f[i][0] = factor(a32, a64, at);
           f[i][1] = factor(a32, a64, at2);
         }
@@ -634,8 +636,12 @@ __global__ void __launch_bounds__(kLineThreads, kLineCtas)
           const int two = 2 * g + 1 < lines;
           const long long bin = base + e + (long long)g * RT;
           const long long lor = lor0 + 2LL * g * R + fdiv((unsigned)at, P.magic_T);
-          x.x *= factor(P.norm32, P.norm, P.norm_per_lor ? lor : bin);
-          x.y *= factor(P.norm32, P.norm, P.norm_per_lor ? lor + two * R : bin + two * RT);
+          const long long n1 = P.norm_per_lor ? dbg_idx(P.dbg, kSiteFinLor, lor, P.n_bins / T)
+                                              : dbg_idx(P.dbg, kSiteFinBin, bin, P.n_bins);
+          const long long n2 = P.norm_per_lor ? dbg_idx(P.dbg, kSiteFinLor, lor + two * R, P.n_bins / T)
+                                              : dbg_idx(P.dbg, kSiteFinBin, bin + two * RT, P.n_bins);
+          x.x *= factor(P.norm32, P.norm, n1);
+          x.y *= factor(P.norm32, P.norm, n2);
         }
       }
       float2* line = rows + g * H.LP;
