@@ -196,14 +196,12 @@ __device__ __forceinline__ void rotate(float3& d, float c, float u) {
     return;
   }
   const float rr = sqrtf(1.0f - d.z * d.z);
-  // the fused operations are written out, so that a direction's last bit does
-  // not depend on which products the compiler chooses to contract
-  float rc;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(rr));
+  // the fused operations and the fast divisions are written out, so that a direction's
+  // last bit does not depend on which products the compiler chooses to contract
   const float tx = __fmul_rn(sn, __fmaf_rn(__fmul_rn(cp, d.x), d.z, -__fmul_rn(sp, d.y)));
   const float ty = __fmul_rn(sn, __fmaf_rn(__fmul_rn(cp, d.y), d.z, __fmul_rn(sp, d.x)));
-  const float nx = __fmaf_rn(c, d.x, __fmul_rn(tx, rc));
-  const float ny = __fmaf_rn(c, d.y, __fmul_rn(ty, rc));
+  const float nx = __fmaf_rn(c, d.x, __fdividef(tx, rr));
+  const float ny = __fmaf_rn(c, d.y, __fdividef(ty, rr));
   const float nz = __fmaf_rn(c, d.z, -__fmul_rn(__fmul_rn(sn, cp), rr));
   d = make_float3(nx, ny, nz);
 }
