@@ -1054,11 +1054,17 @@ static int make_job(psc_ctx* ctx, const psc_sim_args* a, Job& jb, int& lut_dtype
   jb.n = a->n_histories;
   jb.bin_mask = a->bin_mask ? a->bin_mask : PSC_BIN_SCATTER;
   // |z| beyond which a photon that has not interacted is certain to miss the
-  // detector.  The kernel's z of the hit is off the exact line's by at most
-  // about kMaxStraightSteps roundings of the position (2^-23 of the geometry's
-  // scale L each), times tan(incidence), 3 for a grid within 0.95 of the
-  // radius: below 64 * 2^-23 * 3 * 2 L = 5e-5 L.  The margin is L / 512; a grid
-  // nearer to the cylinder gets none (nothing is skipped).
+  // detector.  The kernel reaches the cylinder from a position that kMaxStraightSteps
+  // steps have rounded, each coordinate by at most 2^-24 of its size a step: x and y,
+  // inside the grid, of R, and z of half + zmax; the emission's test and the hit itself
+  // add a few roundings more, 2^-23 a step covers all.  A transverse error moves the chord to
+  // the cylinder by up to 1 / cos(incidence) of itself and the hit's z by the line's slope
+  // times that.  The slope is (|z| + zmax) / chord, and 1 / (chord cos(incidence)) is at
+  // most 1 / (R - rho), 20 / R for a grid within 0.95 of the radius.  So z is off by less than
+  //   64 2^-23 R (20 / R) (half + zmax) + 64 2^-23 (half + zmax) < 1.7e-4 (half + zmax)
+  // however long the scanner or steep the line (beyond the half length |z| grows faster than
+  // its error).  The margin is (R + half + zmax) / 512, twelve times that; a grid nearer to the
+  // cylinder gets none (nothing is skipped).
   {
     const double half = 0.5 * sc->desc.n_rings * sc->desc.ring_pitch;
     const double zmax = std::max(std::fabs(pd.oz), std::fabs(pd.oz + pd.nz * pd.dz));
