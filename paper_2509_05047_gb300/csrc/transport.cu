@@ -36,15 +36,13 @@
 namespace psc {
 
 enum : int {
-  kEmit = 0, kStep = 1, kCompton = 2, kRayleigh = 3, kEscape = 4, kCoinc = 5, kNumSections = 6,
-  kDone = 7
+  kEmit = 0, kStep = 1, kCompton = 2, kRayleigh = 3, kEscape = 4, kCoinc = 5
 };
 
 // Slots per warp: the fuller the sections run, the fewer iterations a history
-// takes.  A model of the pool at the torso's section visits gives 0.204
-// iterations per history at 64 slots, 0.188 at 72 and 0.162 at 96 (0.155 at
-// 128, where every section fills 32 lanes).  96 is what 15 words a slot leave
-// room for beside the tables at 32 warps per SM.
+// takes.  96 is what 15 words a slot leave room for beside the tables at 32
+// warps per SM; with 64 slots of 23 words the paper-scale torso, 1e9 histories,
+// took 88.9 ms (97.8 warp instructions a history), with these 76.1 (65.8).
 constexpr int kSlotsPerWarp = 96;
 constexpr int kSlotsPerLane = kSlotsPerWarp / 32;
 
@@ -95,9 +93,7 @@ enum : int {
 //     ends its history where it leaves the grid, without a detection pass;
 //   - the photon that is less likely to be detected goes first: the one
 //     flying towards the nearer axial end when a line misses, else the one
-//     with the longer way through the phantom.  On the torso 0.16 instead of
-//     0.25 second photons per history, 2.6 instead of 3.1 step visits, 0.33
-//     instead of 0.85 detection visits (counted with the FP64 oracle).
+//     with the longer way through the phantom.
 // Measured on the paper-scale torso, 1e9 histories: 101.7 -> 88.9 ms; the same
 // scanner with gaps and energy resolution, 1e8: 12.32 -> 9.76 ms.
 constexpr uint32_t kMetaNeeds = 1u << 6;     // the photon in flight is lost unless it interacts
@@ -626,7 +622,7 @@ __global__ void __launch_bounds__(512, 2) transport_kernel(const __grid_constant
           s_kc[g] = kc;
         }
 
-        // ---- one Rayleigh try (material id in the upper half of tries) ----
+        // ---- one Rayleigh try (the material travels in meta) ----
         if (sec == kRayleigh) {
           const float u1 = u01(r0), u2 = u01(r1);
           kc.x -= 2u;
