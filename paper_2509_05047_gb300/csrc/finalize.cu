@@ -1275,7 +1275,7 @@ static cudaError_t for_window_radius(int kt, F&& f) {
 static bool line_stage(const FinParams& p, LineStage* h) {
   const int KT = p.KT[0], R = p.R, T = p.T;
   if (KT < 0 || R < KT) return false;
-  if (!radial_lines_pay(T, (long long)finalize_planes(p) * p.V * T, p.K[0], (p.sens_first && p.sens) || p.norm)) return false;
+  if (!radial_lines_pay(T, finalize_planes(p), p.V, p.K[0], (p.sens_first && p.sens) || p.norm)) return false;
   const int RB = (R + 7) / 8, items = RB * T;
   if (items > kLineThreads) return false;
   h->RB = RB;

@@ -35,19 +35,21 @@ inline bool padded_tiles_pay(int radius, AxialForm form, int n_rings, long long 
 // A column's neighbours lie T bins apart, so with few TOF bins a column's loads waste
 // sectors: up to 4 bins lines always pay (448 x 45, radius 8: 1 bin 1798 -> 572 us, 3 bins
 // 2088 -> 1737, 4 bins 0.97 - 0.99 of the whole call).  Above that the column pass is the better one
-// once its columns (planes x views x TOF bins) fill the chip; until then it walks whole lines
-// with too few threads.  Time of the whole call with lines over that with columns, 40 to 448
-// crystals, 5 to 60 TOF bins:
-//   below 75,000 columns: 0.7 - 1.0 (up to 1.11 at 27 bins without smoothing along rad)
-//   up to 200,000: radius 16 and up 0.6 - 0.9, 9 - 12 without a factor 0.7 - 1.0 to 120,000 and
-//     to 1.07 above; below radius 9 0.85 - 1.2 without a factor (worst between 85,000 and
-//     150,000); with a sensitivity or normalisation in the pass, which lines load
-//     together with the counts, 0.5 - 0.98 up to 20 bins, to 1.08 at 27
-inline bool radial_lines_pay(int T, long long columns, int radius, bool factors) {
+// once its columns (planes x views x TOF bins) keep the chip busy; below 200,000 that is so
+// only where its CTAs of 256 columns, each of which walks whole lines, just fill one wave
+// (4 CTAs an SM, 5 up to radius 3, on 152 SMs), for narrow windows without factors (lines load
+// a sensitivity or normalisation together with the counts).  Time of the whole call with
+// lines over that with columns, 40 to 448 crystals, 5 to 60 TOF bins, 1533 calls:
+//   radius up to 8, no factor, one wave filled to more than 0.6: 0.86 - 1.20, 1.03 on average (100 x
+//     10, 27 TOF bins: 109 against 131 us; 300 x 10, 9 bins: 316 against 353)
+//   the others: 0.41 - 1.14, 0.82 on average (more than 1.03 in 34 of 1379)
+inline bool radial_lines_pay(int T, long long planes, int views, int radius, bool factors) {
+  const long long columns = planes * views * T;
   if (T <= 4) return true;
-  if (radius > 12) return columns <= 200000;
-  if (T > 20 || (!factors && radius < 9)) return columns <= 75000;
-  return columns <= (factors ? 200000 : 120000);
+  if (columns > 200000) return false;
+  if (factors || radius > 8) return true;
+  const long long wave = 152 * (radius <= 3 ? 5 : 4), ctas = planes * ((views * T + 255) / 256);
+  return ctas > wave || 5 * columns <= 3 * 256 * wave;
 }
 
 }  // namespace psc

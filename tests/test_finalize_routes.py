@@ -28,11 +28,12 @@ def test_padded_axial_tiles(tmp_path, V, R, T, rings, radius, form, tiles):
     assert _evaluate(tmp_path, [f"padded_tiles_pay({radius}, kAxial{form}, {rings}, {columns}LL)"]) == [tiles]
 
 
-# TOF bins, columns, radius, a factor in the pass: lines slower than columns by 1.04 to 1.2, and faster by 1.1 to 2
-@pytest.mark.parametrize("T,columns,radius,factors,lines", [
-    (27, 135_000, 0, 0, 0), (27, 135_000, 4, 0, 0), (27, 86_400, 2, 0, 0), (27, 135_000, 8, 1, 0), (9, 135_000, 8, 0, 0), (5, 144_000, 4, 0, 0),
-    (13, 93_600, 0, 0, 0), (13, 124_800, 8, 0, 0), (9, 135_000, 12, 0, 0), (9, 230_000, 8, 0, 0), (5, 250_000, 16, 1, 0),
-    (1, 10_000_000, 8, 0, 1), (4, 2_000_000, 24, 1, 1), (7, 14_336, 4, 0, 1), (13, 46_000, 8, 0, 1), (5, 189_280, 8, 1, 1), (9, 163_296, 24, 0, 1),
-    (20, 162_000, 16, 0, 1), (13, 91_000, 12, 0, 1)])
-def test_radial_lines(tmp_path, T, columns, radius, factors, lines):
-    assert _evaluate(tmp_path, [f"radial_lines_pay({T}, {columns}LL, {radius}, {factors})"]) == [lines]
+# crystals, rings, TOF bins, radius, a factor in the pass: lines slower than columns by 1.04 to 1.2, and faster by 1.05 to 2
+@pytest.mark.parametrize("crystals,rings,T,radius,factors,lines", [
+    (100, 10, 27, 4, 0, 0), (100, 10, 27, 8, 0, 0), (300, 10, 9, 8, 0, 0), (100, 24, 5, 4, 0, 0), (100, 15, 13, 0, 0, 0), (200, 10, 13, 8, 0, 0),
+    (200, 16, 9, 8, 0, 0), (448, 20, 5, 16, 1, 0),                                                   # above 200,000 columns
+    (448, 45, 1, 8, 0, 1), (448, 45, 4, 24, 1, 1), (64, 8, 7, 4, 0, 1), (448, 13, 5, 8, 0, 1),      # short TOF axes; few columns; a second wave
+    (40, 16, 27, 8, 0, 1), (40, 44, 5, 8, 0, 1),                                                    # CTAs that are half empty
+    (300, 10, 9, 8, 1, 1), (100, 24, 5, 12, 0, 1), (448, 9, 9, 24, 0, 1), (200, 9, 20, 16, 0, 1)])  # factors, wide windows
+def test_radial_lines(tmp_path, crystals, rings, T, radius, factors, lines):
+    assert _evaluate(tmp_path, [f"radial_lines_pay({T}, {rings * rings}, {crystals // 2}, {radius}, {factors})"]) == [lines]
