@@ -12,23 +12,42 @@ namespace psc {
 // register window; but a CTA sets up barriers, a row table and its copies first,
 // and a tile has one thread for two columns.  So tiles pay for wide windows and
 // where there are many columns (segments x bins of a plane) to hide the set-up.
-// Time of the whole call with tiles over that with the direct pass (8 to 90 rings, planes of
-// 45 to 140,000 bins):
+// So the line is a number of columns for each window, form of the epilogue (a
+// normalisation or its division is one more load an output) and length of the segments
+// (tiles of 37 rows and more are half as wide, those of 90 leave room for few).  Time of the
+// whole call with tiles over that with the direct pass, 8 to 90 rings, planes of 45 to 140,000 bins:
 //   radius 25 - 32: 0.16 - 0.9 everywhere (direct: a load per tap)
-//   radius 16: 0.7 on average above 275,000 columns, 1.3 (up to 1.8) below
-//   radius 9 - 12: 0.8 above 700,000, 1.3 below; with a normalisation or its division (one
-//     more load an output, fewer tiles of more than 48 rows at once) 1.05 - 1.2 at 64 and 90 rings
-//   radius 3 - 8: 0.9 above 700,000 and up to 64 rings (48 with a normalisation), 1.1 - 1.4 below
-//     or at 90 rings; the division 1.1 - 1.6 everywhere
-//   radius 0 - 2: 1.0 at best; with a normalisation 0.9 above 700,000 and up to 48 rings
-enum AxialForm { kAxialPlain, kAxialNorm, kAxialDivide };
+//   radius 13 - 24: 0.4 - 0.95 above the line, 0.9 - 1.9 below
+//   radius 9 - 12: 0.7 - 0.95 and 1.0 - 2.1
+//   radius 3 - 8: 0.8 - 0.98 and 1.0 - 2.2
+//   radius 0 - 2: 0.95 - 1.0 and 1.0 - 1.6; with a normalisation 0.87 - 0.99 and 1.0 - 2.3
+enum AxialForm { kAxialPlain = 0, kAxialNorm = 1, kAxialDivide = 2 };
 
 inline bool padded_tiles_pay(int radius, AxialForm form, int n_rings, long long columns) {
   if (radius > 24) return true;
-  if (radius > 12) return columns >= 275000;
-  if (form == kAxialDivide && radius <= 8) return false;
-  if (form == kAxialPlain && radius <= 2) return false;
-  return columns >= 700000 && n_rings <= (form != kAxialPlain ? 48 : radius > 8 ? 96 : 64);
+  constexpr long long kNever = 1LL << 62;
+  if (n_rings == 1) return radius > 2;
+  // columns from which tiles pay: form, window (radius 0 - 2, 3 - 8, 9 - 12, 13 - 16, 17 - 24), and up
+  // to 8, 36, 48, 64 and more rings
+  constexpr long long kLeast[3][5][5] = {
+      {{6000000, 6000000, kNever, kNever, kNever},
+       {250000, 500000, 800000, 900000, kNever},
+       {150000, 300000, 500000, 450000, 450000},
+       {80000, 150000, 300000, 200000, 110000},
+       {50000, 90000, 155000, 155000, 50000}},
+      {{700000, 700000, 1500000, kNever, kNever},
+       {350000, 550000, 1000000, kNever, kNever},
+       {250000, 400000, 650000, 800000, kNever},
+       {150000, 220000, 275000, 275000, 220000},
+       {80000, 110000, 160000, 160000, 220000}},
+      {{kNever, kNever, kNever, kNever, kNever},
+       {400000, 1900000, 5000000, kNever, kNever},
+       {200000, 300000, 600000, 600000, kNever},
+       {150000, 220000, 275000, 275000, 220000},
+       {80000, 110000, 160000, 160000, 220000}}};
+  const int window = radius <= 2 ? 0 : radius <= 8 ? 1 : radius <= 12 ? 2 : radius <= 16 ? 3 : 4;
+  const int rows = n_rings <= 8 ? 0 : n_rings <= 36 ? 1 : n_rings <= 48 ? 2 : n_rings <= 64 ? 3 : 4;
+  return columns >= kLeast[form][window][rows];
 }
 
 // The radial pass: whole lines staged in shared memory, or a column a thread.

@@ -20,7 +20,7 @@ def _evaluate(tmp_path, expressions):
 @pytest.mark.parametrize("V,R,T,rings,radius,form,tiles", [
     (19, 37, 1, 37, 2, "Plain", 0), (19, 37, 5, 45, 8, "Plain", 0), (51, 101, 1, 37, 8, "Norm", 0), (27, 25, 5, 64, 8, "Norm", 0),
     (51, 101, 5, 90, 8, "Norm", 0), (11, 21, 1, 45, 12, "Norm", 0), (5, 9, 27, 45, 16, "Plain", 0), (11, 21, 5, 37, 16, "Norm", 0),
-    (51, 101, 27, 8, 8, "Divide", 0), (51, 101, 5, 64, 2, "Plain", 0),
+    (51, 101, 5, 16, 8, "Divide", 0), (51, 101, 5, 64, 2, "Plain", 0),
     (51, 101, 27, 45, 8, "Plain", 1), (51, 101, 13, 37, 8, "Norm", 1), (105, 99, 13, 36, 12, "Norm", 1), (51, 101, 13, 45, 16, "Plain", 1),
     (51, 101, 5, 90, 16, "Plain", 1), (5, 9, 1, 8, 25, "Plain", 1), (5, 9, 5, 45, 32, "Divide", 1), (105, 99, 13, 16, 12, "Divide", 1)])
 def test_padded_axial_tiles(tmp_path, V, R, T, rings, radius, form, tiles):
