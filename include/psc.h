@@ -286,7 +286,7 @@ int psc_simulate_batch(psc_ctx* ctx, const psc_sim_args* args, int32_t n, psc_st
 typedef struct {
   int32_t block;            /* threads per CTA */
   int32_t grid;             /* CTAs (0: as many as fit on the device) */
-  int32_t chunks_per_cta;   /* work items per CTA and request, at least */
+  int32_t chunks_per_cta;   /* work items per CTA and request, at least (fewer where items would be too small) */
   int32_t max_chunk;        /* histories per work item at most */
   double rate;              /* histories/s this schedule reached in the probes */
   int32_t probed;           /* schedules timed by this call (0: the choice was cached) */
